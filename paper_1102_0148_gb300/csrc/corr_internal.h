@@ -103,6 +103,10 @@ struct FengineArgs {
 };
 
 cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st);
+// The kernels with a tensor-core first stage (fengine_mma.cu), and whether
+// they serve these arguments (K, output type, input alignment).
+bool fengine_mma_serves(const FengineArgs& a);
+cudaError_t launch_fengine_mma(const FengineArgs& a, cudaStream_t st);
 // The F-engines of n modes (1 <= n <= 4, one workspace element type, no
 // debug output) as one launch: each mode's frames as its own kernel would
 // transform them.

@@ -392,26 +392,6 @@ __device__ __forceinline__ void group_bar(int id, int n) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// 8-point forward DFT in place (radix 2 x 4).
-__device__ __forceinline__ void dft8(float2& x0, float2& x1, float2& x2, float2& x3, float2& x4,
-                                     float2& x5, float2& x6, float2& x7) {
-    constexpr float r2 = 0.707106781186547524f;
-    dft4(x0, x2, x4, x6);                         // E[0..3] in x0, x2, x4, x6
-    dft4(x1, x3, x5, x7);                         // O[0..3] in x1, x3, x5, x7
-    const float2 o1 = make_float2(r2 * (x3.x + x3.y), r2 * (x3.y - x3.x));    // W8^1 O1
-    const float2 o2 = cmi(x5);                                                // W8^2 O2
-    const float2 o3 = make_float2(r2 * (x7.y - x7.x), -r2 * (x7.x + x7.y));   // W8^3 O3
-    const float2 e0 = x0, e1 = x2, e2 = x4, e3 = x6, o0 = x1;
-    x0 = cadd(e0, o0);
-    x4 = csub(e0, o0);
-    x1 = cadd(e1, o1);
-    x5 = csub(e1, o1);
-    x2 = cadd(e2, o2);
-    x6 = csub(e2, o2);
-    x3 = cadd(e3, o3);
-    x7 = csub(e3, o3);
-}
-
 template <int R>
 __device__ __forceinline__ void dft_r(float2 (&v)[R]) {
     if constexpr (R == 4) {
@@ -721,7 +701,10 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
     const int L = a.K / 2;
     const int C = L;
     const bool dbg = a.debug_out != nullptr;
-    // K = 512 with 16-byte aligned input (the fast kernel reads 16 B per lane).
+    if (fengine_mma_serves(a)) return launch_fengine_mma(a, st);
+    // K = 512 with 16-byte aligned input (the kernel reads 16 B per lane): the
+    // FP32 and FP16-pair outputs, bound by their own bytes (350 us per 16384
+    // frames at N = 44 in FP32 mode either way)
     if (a.K == 512 && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
         const int64_t fr = dbg ? a.S : a.S_pad;
         if (fr <= 0) return cudaSuccess;
@@ -730,11 +713,9 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         b.ant_x = nfb <= 65535;
         const dim3 grid = b.ant_x ? dim3((unsigned)a.N, (unsigned)nfb) : dim3((unsigned)nfb, (unsigned)a.N);
         // staging (also the exchange areas), the twiddle bases, and when used
-        // the scales and the corrections, for the debug output too (at most
-        // 72 KB: three CTAs per SM)
-        const bool scaled = !dbg && (a.spec_type == SPEC_F16 || a.spec_type == SPEC_F8);
+        // the corrections, for the debug output too (at most 72 KB: three CTAs
+        // per SM)
         const size_t smem = (size_t)kStgFloats * sizeof(float) + 128 * sizeof(float2) +
-                            (scaled ? 256 * sizeof(float) : 0) +
                             (a.corr ? 256 * sizeof(float2) : 0);
         auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -747,8 +728,6 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         if (dbg) return go2(fengine_k512<kOutDebug, false>, fengine_k512<kOutDebug, true>);
         switch (a.spec_type) {
             case SPEC_F32: return go2(fengine_k512<SPEC_F32, false>, fengine_k512<SPEC_F32, true>);
-            case SPEC_F16: return go2(fengine_k512<SPEC_F16, false>, fengine_k512<SPEC_F16, true>);
-            case SPEC_F8: return go2(fengine_k512<SPEC_F8, false>, fengine_k512<SPEC_F8, true>);
             default: return go2(fengine_k512<SPEC_F16X2, false>, fengine_k512<SPEC_F16X2, true>);
         }
     }
@@ -761,13 +740,8 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         b.ant_x = 0;
         const dim3 grid((unsigned)nfb, (unsigned)a.N);
         // staging (also the exchange areas) and the twiddle tables, for the
-        // debug output too
-        // staging (also the exchange areas), the twiddle tables and for
-        // FP16/FP8 the scales, for the debug output too (at most 71 KB: three
-        // CTAs per SM)
-        const bool scaled = !dbg && (a.spec_type == SPEC_F16 || a.spec_type == SPEC_F8);
-        const size_t smem = (size_t)kStg1024Floats * sizeof(float) + (256 + 32) * sizeof(float2) +
-                            (scaled ? 512 * sizeof(float) : 0);
+        // debug output too (at most 70 KB: three CTAs per SM)
+        const size_t smem = (size_t)kStg1024Floats * sizeof(float) + (256 + 32) * sizeof(float2);
         auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem);
@@ -779,40 +753,29 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         if (dbg) return go2(fengine_k1024<kOutDebug, false>, fengine_k1024<kOutDebug, true>);
         switch (a.spec_type) {
             case SPEC_F32: return go2(fengine_k1024<SPEC_F32, false>, fengine_k1024<SPEC_F32, true>);
-            case SPEC_F16: return go2(fengine_k1024<SPEC_F16, false>, fengine_k1024<SPEC_F16, true>);
-            case SPEC_F8: return go2(fengine_k1024<SPEC_F8, false>, fengine_k1024<SPEC_F8, true>);
             default: return go2(fengine_k1024<SPEC_F16X2, false>, fengine_k1024<SPEC_F16X2, true>);
         }
     }
-    if ((a.K == 2048 || a.K == 4096) && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
+    if (a.K == 4096 && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
         const int64_t fr = dbg ? a.S : a.S_pad;
         if (fr <= 0) return cudaSuccess;
-        auto go = [&](auto kern, int FT, size_t smem) -> cudaError_t {
+        using Sh = Rad16Shape<8>;
+        const size_t smem = Sh::smem(dbg);
+        auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem);
             if (e != cudaSuccess) return e;
-            dim3 grid((unsigned)((fr + FT - 1) / FT), (unsigned)a.N);
+            dim3 grid((unsigned)((fr + Sh::FT - 1) / Sh::FT), (unsigned)a.N);
             kern<<<grid, kRadThreads, smem, st>>>(a);
             return cudaGetLastError();
         };
-        auto pick = [&](auto shape, auto k_dbg, auto k_f32, auto k_f16, auto k_f8, auto k_x2) {
-            using Sh = decltype(shape);
-            const size_t sm = Sh::smem(dbg);
-            if (dbg) return go(k_dbg, Sh::FT, sm);
-            switch (a.spec_type) {
-                case SPEC_F32: return go(k_f32, Sh::FT, sm);
-                case SPEC_F16: return go(k_f16, Sh::FT, sm);
-                case SPEC_F8: return go(k_f8, Sh::FT, sm);
-                default: return go(k_x2, Sh::FT, sm);
-            }
-        };
-        if (a.K == 2048)
-            return pick(Rad16Shape<4>{}, fengine_rad16<4, kOutDebug>, fengine_rad16<4, SPEC_F32>,
-                        fengine_rad16<4, SPEC_F16>, fengine_rad16<4, SPEC_F8>,
-                        fengine_rad16<4, SPEC_F16X2>);
-        return pick(Rad16Shape<8>{}, fengine_rad16<8, kOutDebug>, fengine_rad16<8, SPEC_F32>,
-                    fengine_rad16<8, SPEC_F16>, fengine_rad16<8, SPEC_F8>,
-                    fengine_rad16<8, SPEC_F16X2>);
+        if (dbg) return go(fengine_rad16<8, kOutDebug>);
+        switch (a.spec_type) {
+            case SPEC_F32: return go(fengine_rad16<8, SPEC_F32>);
+            case SPEC_F16: return go(fengine_rad16<8, SPEC_F16>);
+            case SPEC_F8: return go(fengine_rad16<8, SPEC_F8>);
+            default: return go(fengine_rad16<8, SPEC_F16X2>);
+        }
     }
     int FT = 8192 / C;
     FT = FT < 1 ? 1 : (FT > 32 ? 32 : FT);

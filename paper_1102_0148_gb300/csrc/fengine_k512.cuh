@@ -99,6 +99,26 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
     for (int q = 0; q < 16; ++q) x[q] = y[q];
 }
 
+// 8-point forward DFT in place (radix 2 x 4).
+__device__ __forceinline__ void dft8(float2& x0, float2& x1, float2& x2, float2& x3, float2& x4,
+                                     float2& x5, float2& x6, float2& x7) {
+    constexpr float r2 = 0.707106781186547524f;
+    dft4(x0, x2, x4, x6);                         // E[0..3] in x0, x2, x4, x6
+    dft4(x1, x3, x5, x7);                         // O[0..3] in x1, x3, x5, x7
+    const float2 o1 = make_float2(r2 * (x3.x + x3.y), r2 * (x3.y - x3.x));    // W8^1 O1
+    const float2 o2 = cmi(x5);                                                // W8^2 O2
+    const float2 o3 = make_float2(r2 * (x7.y - x7.x), -r2 * (x7.x + x7.y));   // W8^3 O3
+    const float2 e0 = x0, e1 = x2, e2 = x4, e3 = x6, o0 = x1;
+    x0 = cadd(e0, o0);
+    x4 = csub(e0, o0);
+    x1 = cadd(e1, o1);
+    x5 = csub(e1, o1);
+    x2 = cadd(e2, o2);
+    x6 = csub(e2, o2);
+    x3 = cadd(e3, o3);
+    x7 = csub(e3, o3);
+}
+
 // Nibble v (0..15, 4-bit two's complement) to float without a conversion
 // instruction: the bit pattern 0x4B000000 | u is the float 2^23 + u.  The
 // high nibble is masked in place (u = 16 (v ^ 8)) and scaled back by the
