@@ -12,6 +12,7 @@
 
 #include <cuda.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -55,7 +56,7 @@ CtxGetCurrentFn ctx_get_current() {
     return fn;
 }
 
-constexpr int64_t kSplit = 256;     // fewest frames per X-engine split (sizes the partials)
+constexpr int64_t kSplit = 256;     // frames per X-engine split when sizing a pass
 constexpr int64_t kMaxPass = 2048;  // frames per pass at most
 
 size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -141,13 +142,22 @@ extern "C" int corr_correlate_noalloc(const uint8_t* samples, int64_t n, int N, 
 
     const int C = K / 2;
     const int P = N * (N + 1) / 2;
-    const int max_split = (int)((S_pass + kSplit - 1) / kSplit);
+    // Partial slots: whatever the pass leaves of the array, one per 32-frame
+    // tile at most.  The pass of 256 frames that fits at N = 44, K = 512 has
+    // only 86 X-engine CTAs (3 channels each) without splits, on 152 SMs, each
+    // a serial chain of 256 frames; with three splits its X-engine takes
+    // 27 us instead of 35.5 (a 2048-frame call 445 -> 364 us).
+    const size_t part_bytes = al256((size_t)C * P * sizeof(float2));
+    const size_t fixed = al256((size_t)K * sizeof(float2)) + al256((size_t)C * P * sizeof(double2)) +
+                         al256((size_t)C * 2 * (size_t)N * (size_t)S_pass * sizeof(float));
+    const int max_split = (int)std::max<int64_t>(
+        1, std::min<int64_t>(S_pass / 32, (int64_t)((kScratchBytes - fixed) / part_bytes)));
     float2* tw = reinterpret_cast<float2*>(base);
     double2* acc = reinterpret_cast<double2*>(base + al256((size_t)K * sizeof(float2)));
     float2* part = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(acc) +
                                              al256((size_t)C * P * sizeof(double2)));
     float* spec = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(part) +
-                                           al256((size_t)max_split * C * P * sizeof(float2)));
+                                           max_split * part_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     // The array keeps the previous call's contents: clear the accumulator.
