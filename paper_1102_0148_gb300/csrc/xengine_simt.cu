@@ -14,9 +14,14 @@
 // (4 antennas x Re, Im) sit in rows 8 b .. 8 b + 7; a row's 16-byte groups
 // (4 frames each) are XOR-swizzled by b mod 8, so the quarter-warp that reads
 // one group of 8 different blocks hits 8 different bank groups.  A thread
-// reads two frames of a row as one float2 and accumulates them with packed
-// FP32 FMAs (FFMA2: even frames in .x, odd frames in .y, summed at the end),
-// half the instructions of scalar FMAs for the same arithmetic.
+// reads a row's group with one 16-byte load and accumulates even and odd
+// frames apart (.x, .y, summed at the end) with scalar FMAs.  What bounds it:
+// issue (70%, a quarter of it copy addresses and loop control) at 14 warps per
+// SM, FP32 pipe 53%, L1 56%.  With 8-byte loads (two frames) and packed FMAs,
+// which run at 2.6 lanes' worth per clock and SM for three distinct operands,
+// the same sums took longer: N = 44, K = 512, 8192 frames 544 -> 508 us,
+// N = 256, K = 1024, 1024 frames 4161 -> 3879, N = 512, K = 64, 2048 frames
+// 3094 -> 2381.
 #include "corr_internal.h"
 
 #include <algorithm>
@@ -30,6 +35,13 @@ constexpr int kMaxStages = 3;    // stages in flight per CTA
 __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+// (ar, ai) += x conj(y)
+__device__ __forceinline__ void cmac(float xr, float xi, float yr, float yi, float& ar, float& ai) {
+    ar = fmaf(xr, yr, ar);
+    ar = fmaf(xi, yi, ar);
+    ai = fmaf(xi, yr, ai);
+    ai = fmaf(-xr, yi, ai);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -74,8 +86,8 @@ __global__ void __launch_bounds__(256) xengine_simt_kernel(XengineArgs a, int nb
                 for (int e = 2 * N * tf + threadIdx.x; e < tile_floats; e += blockDim.x) tg[e] = 0.f;
             }
 
-    // packed pairs: .x sums the even frames, .y the odd ones (one FFMA2 does
-    // both), added together at the end
+    // .x sums the even frames, .y the odd ones,
+    // added together at the end
     float2 ar[4][4], ai[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -125,28 +137,22 @@ __global__ void __launch_bounds__(256) xengine_simt_kernel(XengineArgs a, int nb
             const int swi = bi & gmask, swj = bj & gmask;
 #pragma unroll 1
             for (int c = 0; c <= gmask; ++c) {
+                // rows 2u (Re) and 2u + 1 (Im) of antennas 4 bi + u and 4 bj + v,
+                // frames 4c .. 4c + 3: one 16-byte load per row
+                float4 X[8];
 #pragma unroll
-                for (int f2 = 0; f2 < 4; f2 += 2) {
-                    // rows 2u (Re) and 2u + 1 (Im) of antennas 4 bi + u and
-                    // 4 bj + u, frames 4c + f2 and 4c + f2 + 1
-                    float2 X[8], Y[8];
+                for (int q = 0; q < 8; ++q)
+                    X[q] = *reinterpret_cast<const float4*>(pi + q * tf + ((c ^ swi) << 2));
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        X[q] = *reinterpret_cast<const float2*>(pi + q * tf + ((c ^ swi) << 2) + f2);
-                        Y[q] = *reinterpret_cast<const float2*>(pj + q * tf + ((c ^ swj) << 2) + f2);
-                    }
+                for (int v = 0; v < 4; ++v) {
+                    const float4 yr = *reinterpret_cast<const float4*>(pj + 2 * v * tf + ((c ^ swj) << 2));
+                    const float4 yi = *reinterpret_cast<const float4*>(pj + (2 * v + 1) * tf + ((c ^ swj) << 2));
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const float2 xr = X[2 * u], xi = X[2 * u + 1];
-                        const float2 nxr = make_float2(-xr.x, -xr.y);
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            const float2 yr = Y[2 * v], yi = Y[2 * v + 1];
-                            ar[u][v] = __ffma2_rn(xr, yr, ar[u][v]);
-                            ar[u][v] = __ffma2_rn(xi, yi, ar[u][v]);
-                            ai[u][v] = __ffma2_rn(xi, yr, ai[u][v]);
-                            ai[u][v] = __ffma2_rn(nxr, yi, ai[u][v]);
-                        }
+                        cmac(X[2 * u].x, X[2 * u + 1].x, yr.x, yi.x, ar[u][v].x, ai[u][v].x);
+                        cmac(X[2 * u].y, X[2 * u + 1].y, yr.y, yi.y, ar[u][v].y, ai[u][v].y);
+                        cmac(X[2 * u].z, X[2 * u + 1].z, yr.z, yi.z, ar[u][v].x, ai[u][v].x);
+                        cmac(X[2 * u].w, X[2 * u + 1].w, yr.w, yi.w, ar[u][v].y, ai[u][v].y);
                     }
                 }
             }
