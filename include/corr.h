@@ -99,7 +99,8 @@ int corr_create(corr_t* out, int N, int K, int dtype);
 
 /* Queue later work on `stream` (a cudaStream_t of the handle's device; NULL
  * means the legacy default stream).  Waits for the handle's queued work
- * first. */
+ * first (when the stream is the handle's already, nothing changes and there
+ * is nothing to wait for). */
 int corr_set_stream(corr_t h, void* stream);
 
 /* Capacity of the spectra workspace in frames, rounded up to a multiple of

@@ -69,6 +69,12 @@ struct corr_s {
     float2* partial = nullptr;   // [max_split][C][P]
     int max_split = 0;
     int* status = nullptr;       // device-side error word
+    // page-locked host memory: the status word's copy, and the corrections as
+    // last uploaded (gains, delays, pre-scales; corr_pin_free follows the
+    // copies that read them)
+    int* status_host = nullptr;
+    float* corr_pin = nullptr;
+    cudaEvent_t corr_pin_free = nullptr;
     // host-input staging ring: copies run ahead of the F-engine by up to
     // kHostStages - 1 chunks of stage_frames frames
     uint8_t* stage[kHostStages] = {};
@@ -206,15 +212,32 @@ int alloc_workspace(corr_t h, int64_t cap) {
     return CORR_OK;
 }
 
-int check_status(corr_t h) {
-    int st = 0;
-    CUDA_TRY(h, cudaMemcpy(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost));
+// Queue the copy of the status word behind the handle's work; read_status
+// inspects it once the stream has been waited for.  (One wait for the work and
+// the word: a blocking copy after the wait cost another round trip, ~8 us of a
+// 70 us call.)
+int queue_status(corr_t h) {
+    CUDA_TRY(h, cudaMemcpyAsync(h->status_host, h->status, sizeof(int), cudaMemcpyDeviceToHost,
+                                h->stream));
+    return CORR_OK;
+}
+
+int read_status(corr_t h) {
+    const int st = *static_cast<volatile int*>(h->status_host);
     if (st != 0) {
         CUDA_TRY(h, cudaMemset(h->status, 0, sizeof(int)));
         if (h->tc) tc_reset(h->tc);
         return set_err(h, CORR_ETIMEOUT, "a bounded device-side wait gave up (code %d)", st);
     }
     return CORR_OK;
+}
+
+// Wait for the handle's stream and report device-side errors.
+int wait_and_check(corr_t h) {
+    int rc = queue_status(h);
+    if (rc != CORR_OK) return rc;
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return read_status(h);
 }
 
 cudaEvent_t prof_event(corr_t h) {
@@ -649,6 +672,9 @@ void destroy_impl(corr_t h) {
     cudaFree(h->grad_buf);
     cudaFree(h->grad_scratch);
     cudaFree(h->status);
+    cudaFreeHost(h->status_host);
+    cudaFreeHost(h->corr_pin);
+    if (h->corr_pin_free) cudaEventDestroy(h->corr_pin_free);
     cudaFree(h->vis_dev);
     cudaFree(h->sdelay);
     cudaFree(h->hist[0]);
@@ -747,8 +773,15 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
         if (cudaStreamCreateWithFlags(&h->f_stream[j], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->f_done[j], cudaEventDisableTiming) != cudaSuccess)
             return bail(set_err(h, CORR_ECUDA, "stream creation failed"));
-    if (cudaEventCreateWithFlags(&h->f_fork, cudaEventDisableTiming) != cudaSuccess)
+    if (cudaEventCreateWithFlags(&h->f_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->corr_pin_free, cudaEventDisableTiming) != cudaSuccess)
         return bail(set_err(h, CORR_ECUDA, "event creation failed"));
+    if (cudaMallocHost((void**)&h->status_host, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost((void**)&h->corr_pin, 4 * (size_t)N * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        return bail(set_err(h, CORR_ENOMEM, "host allocation failed"));
+    }
+    *h->status_host = 0;
     h->f_last = h->stream;
 
     if (h->use_tc) {
@@ -820,6 +853,7 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
 
 int corr_set_stream(corr_t h, void* stream) {
     if (!h) return CORR_EINVAL;
+    if (!h->own_stream && h->stream == static_cast<cudaStream_t>(stream)) return CORR_OK;
     int frc = fx_flush(h);
     if (frc != CORR_OK) return frc;
     int jrc = join_fengines(h);
@@ -941,8 +975,7 @@ int corr_save_state(corr_t h, void* buf) {
     int frc = flush(h);
     if (frc == CORR_OK) frc = settle_partial(h);
     if (frc != CORR_OK) return frc;
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    int rc = check_status(h);
+    int rc = wait_and_check(h);
     if (rc != CORR_OK) return rc;
     StateHeader hd{kStateMagic, h->N, h->K, h->dtype, h->scales_ready ? 1 : 0, h->n_spec,
                    h->sdelay_on ? 1 : 0, 0};
@@ -1045,11 +1078,19 @@ int corr_set_sample_delays(corr_t h, const int32_t* delays) {
 
 int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
     if (!h) return CORR_EINVAL;
-    // Host copies, to check the values and to derive the two-plane pre-scales.
-    std::vector<float> gh, th;
-    if (gains) {
-        gh.resize(2 * (size_t)h->N);
-        CUDA_TRY(h, cudaMemcpy(gh.data(), gains, gh.size() * sizeof(float), cudaMemcpyDefault));
+    // Host copies in page-locked memory, to check the values, to derive the
+    // two-plane pre-scales and to upload from: one wait for both inputs, none
+    // for the uploads.  (The copies go through the legacy default stream, whose
+    // ordering a blocking cudaMemcpy has.)
+    CUDA_TRY(h, cudaEventSynchronize(h->corr_pin_free));   // the previous call's uploads
+    float* gh = h->corr_pin;
+    float* th = gh + 2 * (size_t)h->N;
+    if (gains)
+        CUDA_TRY(h, cudaMemcpyAsync(gh, gains, (size_t)h->N * sizeof(float2), cudaMemcpyDefault, 0));
+    if (delays)
+        CUDA_TRY(h, cudaMemcpyAsync(th, delays, (size_t)h->N * sizeof(float), cudaMemcpyDefault, 0));
+    if (gains || delays) CUDA_TRY(h, cudaStreamSynchronize(0));
+    if (gains)
         for (int i = 0; i < h->N; ++i) {
             const double a = std::hypot((double)gh[2 * i], (double)gh[2 * i + 1]);
             if (!std::isfinite(a) || a > kGainMax || (a > 0.0 && a < kGainMin))
@@ -1057,14 +1098,10 @@ int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
                                "gain %d has modulus %g: gains must be finite, 0 or within "
                                "[2^-40, 2^40]", i, a);
         }
-    }
-    if (delays) {
-        th.resize(h->N);
-        CUDA_TRY(h, cudaMemcpy(th.data(), delays, th.size() * sizeof(float), cudaMemcpyDefault));
+    if (delays)
         for (int i = 0; i < h->N; ++i)
             if (!std::isfinite(th[i]))
                 return set_err(h, CORR_EINVAL, "delay %d is not finite", i);
-    }
     // launches already queued keep the old tables; pushes waiting for the
     // fused launch are run with them now
     int frc0 = fx_flush(h);
@@ -1085,9 +1122,11 @@ int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
             if (frc != CORR_OK) return frc;
         }
         if (sn != h->split_host) {
-            CUDA_TRY(h, cudaMemcpyAsync(h->split + h->N, sn.data(), h->N * sizeof(float),
+            float* sh = th + h->N;
+            std::copy(sn.begin(), sn.end(), sh);
+            CUDA_TRY(h, cudaMemcpyAsync(h->split + h->N, sh, h->N * sizeof(float),
                                         cudaMemcpyHostToDevice, h->stream));
-            CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+            CUDA_TRY(h, cudaEventRecord(h->corr_pin_free, h->stream));
             h->split_host = sn;
         }
     }
@@ -1096,15 +1135,15 @@ int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
         return CORR_OK;
     }
     if (gains)
-        CUDA_TRY(h, cudaMemcpyAsync(h->gains_dev, gains, (size_t)h->N * sizeof(float2),
-                                    cudaMemcpyDefault, h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(h->gains_dev, gh, (size_t)h->N * sizeof(float2),
+                                    cudaMemcpyHostToDevice, h->stream));
     if (delays)
-        CUDA_TRY(h, cudaMemcpyAsync(h->delays_dev, delays, (size_t)h->N * sizeof(float),
-                                    cudaMemcpyDefault, h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(h->delays_dev, th, (size_t)h->N * sizeof(float),
+                                    cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(h, cudaEventRecord(h->corr_pin_free, h->stream));
     CUDA_TRY(h, launch_correction_table(gains ? h->gains_dev : nullptr,
                                         delays ? h->delays_dev : nullptr, h->N, h->K, h->corr_tab,
                                         h->stream));
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     h->corr_on = true;
     return CORR_OK;
 }
@@ -1170,8 +1209,7 @@ int corr_grad(corr_t h, const uint8_t* samples, int64_t n, const float* gains,
                                 h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(grad_delays, gt_dev, h->N * sizeof(float), cudaMemcpyDefault,
                                 h->stream));
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    return check_status(h);
+    return wait_and_check(h);
 }
 
 namespace {
@@ -1225,8 +1263,10 @@ int corr_dump(corr_t h, void* vis, int64_t* n_spec, int vis_fp64) {
     if (!vis) return set_err(h, CORR_EINVAL, "vis is NULL");
     int rc = enqueue_dump(h, vis, vis_fp64, is_device_ptr(vis));
     if (rc != CORR_OK) return rc;
+    rc = queue_status(h);
+    if (rc != CORR_OK) return rc;
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    rc = check_status(h);
+    rc = read_status(h);
     if (n_spec) *n_spec = h->n_spec;
     h->n_spec = 0;
     return rc;
@@ -1254,8 +1294,7 @@ int corr_sync(corr_t h) {
     if (!h) return CORR_EINVAL;
     int frc = flush(h);
     if (frc != CORR_OK) return frc;
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    return check_status(h);
+    return wait_and_check(h);
 }
 
 void corr_destroy(corr_t h) { destroy_impl(h); }
@@ -1649,10 +1688,14 @@ int corr_batch_replay(corr_batch_t b, int64_t* n_spec) {
 
 int corr_batch_sync(corr_batch_t b) {
     if (!b) return CORR_EINVAL;
+    for (int m = 0; m < b->n; ++m) {             // one wait for all the modes' status words
+        int rc = queue_status(b->h[m]);
+        if (rc != CORR_OK) return batch_from_handle(b, m, rc);
+    }
     if (cudaStreamSynchronize(b->stream) != cudaSuccess)
         return batch_err(b, CORR_ECUDA, cudaGetErrorString(cudaGetLastError()));
     for (int m = 0; m < b->n; ++m) {
-        int rc = check_status(b->h[m]);
+        int rc = read_status(b->h[m]);
         if (rc != CORR_OK) return batch_from_handle(b, m, rc);
     }
     return CORR_OK;
