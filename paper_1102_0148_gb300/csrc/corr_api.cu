@@ -436,6 +436,7 @@ int xengine_pass(corr_t h, int64_t S_pad, double2* acc) {
         run.scale = h->scale;
         run.split = h->fill_split;
         run.status = h->status;
+        run.assign = acc == h->acc && h->acc_zero;
         TcPlan* plans[1] = {h->tc};
         int rc = tc_launch(plans, 1, &run, h->stream, h->err);
         if (rc != CORR_OK) return rc;
@@ -1486,6 +1487,7 @@ int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* 
             r.scale = h->scale;
             r.split = split_table(h, false);
             r.status = h->status;
+            r.assign = h->acc_zero;
             plans[na] = h->tc;
             runs[na] = r;
             idx[na++] = m;

@@ -81,6 +81,7 @@ struct TcModeArgs {
     int* ticket;              // [C][npairs] arrival counters (n_split > 1), zero between launches
     const float* scale;       // [N][C] pre-cast scales (modes 1, 2)
     const float* split;       // [N] two-plane pre-scales sigma_i (mode 0)
+    int assign;               // acc is known to hold zeros: store instead of adding
 };
 
 struct TcArgs {
@@ -92,13 +93,14 @@ struct TcArgs {
     int atoms;                // k-tiles of KT spectra per pipeline stage
     int row_bytes;            // bytes of one tile row: 64 (FP16 modes) or 128 (FP8)
     int wide;                 // a mode has several antenna blocks: atoms hold A, B0, B1 slots
-    int gs_floats;            // epilogue G buffer (largest 2nb x (2nb + 1) of the modes)
+    int gs_floats;            // epilogue G buffer (largest 2nb x (2nb + 1) of the modes; FP32 mode + 2 kRows)
     int slot_rows;            // rows of one operand tile slot in shared memory (<= 128)
     int* status;
     unsigned long long timeout_ns;
     int withhold;             // test hook: CTA 0 does not load its first k-tile
     int balanced;             // 1: contiguous deal of weighted k-tiles; 0: round-robin items
     int64_t units;            // total work units of the balanced deal
+    int u32;                  // units times CTAs fit 32 bits: cheap divisions
 };
 
 struct Item {
@@ -187,15 +189,23 @@ struct PieceCursor {
     int64_t ibase, lo, hi;
 };
 
-__device__ __forceinline__ int64_t ceil_div64(int64_t x, int64_t y) { return (x + y - 1) / y; }
+// x / y for non-negative operands of the balanced deal.  The cursors divide
+// several times per piece, on one lane and before its first load: ~150 clocks
+// each in 64 bits, a few in 32.
+__device__ __forceinline__ int64_t deal_div(const TcArgs& a, int64_t x, int64_t y) {
+    return a.u32 ? (int64_t)((uint32_t)x / (uint32_t)y) : x / y;
+}
+__device__ __forceinline__ int64_t ceil_div(const TcArgs& a, int64_t x, int64_t y) {
+    return deal_div(a, x + y - 1, y);
+}
 
 __device__ __forceinline__ void cursor_init(const TcArgs& a, PieceCursor& c) {
     c.g = blockIdx.x;
     c.m = a.n_modes;
     if (!a.balanced) return;
     const int64_t G = gridDim.x;
-    c.lo = ceil_div64((int64_t)blockIdx.x * a.units, G);
-    c.hi = ceil_div64((int64_t)(blockIdx.x + 1) * a.units, G);
+    c.lo = ceil_div(a, (int64_t)blockIdx.x * a.units, G);
+    c.hi = ceil_div(a, (int64_t)(blockIdx.x + 1) * a.units, G);
     for (int m = 0; m < a.n_modes; ++m) {
         const TcModeArgs& d = a.md[m];
         int64_t base = d.unit_base;
@@ -205,7 +215,7 @@ __device__ __forceinline__ void cursor_init(const TcArgs& a, PieceCursor& c) {
             if (c.lo < base + pu) {
                 c.m = m;
                 c.pr = pr;
-                c.k = (int)((c.lo - base) / iu);
+                c.k = (int)deal_div(a, c.lo - base, iu);
                 c.ibase = base + (int64_t)c.k * iu;
                 return;
             }
@@ -231,8 +241,8 @@ __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piec
         const TcModeArgs& d = a.md[c.m];
         const int w = pair_units(c.pr, d.nblk);
         const int64_t t0 = c.ibase + kEndUnits;          // first unit of k-tile 0
-        const int64_t j0 = c.lo > t0 ? ceil_div64(c.lo - t0, w) : 0;
-        const int64_t j1 = c.hi > t0 ? min(d.tiles, ceil_div64(c.hi - t0, w)) : 0;
+        const int64_t j0 = c.lo > t0 ? ceil_div(a, c.lo - t0, w) : 0;
+        const int64_t j1 = c.hi > t0 ? min(d.tiles, ceil_div(a, c.hi - t0, w)) : 0;
         const bool mine = j0 < j1;
         if (mine) {
             p.itm.m = c.m;
@@ -243,8 +253,8 @@ __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piec
             const int64_t KT = a.KT;
             p.s_beg = j0 * KT;
             p.s_end = j1 * KT;
-            const int first = (int)(t0 * G / a.units);
-            const int last = (int)((t0 + (d.tiles - 1) * w) * G / a.units);
+            const int first = (int)deal_div(a, t0 * G, a.units);
+            const int last = (int)deal_div(a, (t0 + (d.tiles - 1) * w) * G, a.units);
             p.slot = (int)blockIdx.x - first;
             p.nslots = last - first + 1;
         }
@@ -259,6 +269,18 @@ __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piec
         if (mine) return true;
     }
     return false;
+}
+
+// Upper triangle of n antennas, row-major with autos: first pair of row i, and
+// the row of pair pl.
+__device__ __forceinline__ int triangle_start(int i, int n) { return i * n - i * (i - 1) / 2; }
+__device__ __forceinline__ int triangle_row(int pl, int n) {
+    const float b = 2.0f * n + 1.0f;
+    int i = (int)(0.5f * (b - sqrtf(b * b - 8.0f * pl)));
+    i = min(max(i, 0), n - 1);
+    while (pl < triangle_start(i, n)) --i;             // the root is rounded: at most a step off
+    while (i + 1 < n && pl >= triangle_start(i + 1, n)) ++i;
+    return i;
 }
 
 // Bounded wait with this launch's limit and status word.
@@ -347,8 +369,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
     PieceCursor* epi_cur = reinterpret_cast<PieceCursor*>(
         (reinterpret_cast<uintptr_t>(epi_last + 2) + 15) & ~(uintptr_t)15);
     Piece* epi_pc = reinterpret_cast<Piece*>(epi_cur + 1);
-    volatile int* epi_more = reinterpret_cast<volatile int*>(epi_pc + 1);
-    volatile int* epi_abort = epi_more + 1;
+    volatile int* epi_more = reinterpret_cast<volatile int*>(epi_pc + 2);   // [2], as epi_pc
+    volatile int* epi_abort = epi_more + 2;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -556,16 +578,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         const int r = 32 * q + lane;
         int wi = 0;
         // one cursor for the 8 warps, in shared memory (registers are scarce here)
-        if (et == 0) cursor_init(a, *epi_cur);
-        for (;;) {
-            if (et == 0) *epi_more = next_piece(a, *epi_cur, *epi_pc) ? 1 : 0;
-            epi_sync();
-            if (!*epi_more) break;
-            const Piece pc = *epi_pc;
+        if (et == 0) {
+            cursor_init(a, *epi_cur);
+            epi_more[0] = next_piece(a, *epi_cur, epi_pc[0]) ? 1 : 0;
+        }
+        epi_sync();
+        for (int pb = 0;; pb ^= 1) {
+            if (!epi_more[pb]) break;
+            const Piece pc = epi_pc[pb];
+            // the piece after it, while this one's windows are on their way
+            if (et == 0) epi_more[pb ^ 1] = next_piece(a, *epi_cur, epi_pc[pb ^ 1]) ? 1 : 0;
             const Item& itm = pc.itm;
             const TcModeArgs& d = a.md[itm.m];
             const bool single = !WIDE || d.nblk == 1;
-            const bool diag = single;                // the single block's pair (b1 = b2 = 0)
             const bool use_t = MODE == 0 && single;
             const int nb1 = block_ants(d.N, itm.b1);
             const int nb2 = single ? nb1 : block_ants(d.N, itm.b2);
@@ -694,32 +719,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     }
                 }
             } else {
+            // FP32 mode: G = S + L^T with S = Dhh + Dhl and L = Dhl.  Only the
+            // 2 x 2 antenna blocks on and above the diagonal are needed, so
+            // the square holds S there and L below it, and L of the diagonal
+            // blocks has its own place (Ld): one store per element, and the
+            // pair adds the transposed element when it reads.  (Adding L^T in
+            // place cost a dependent shared load, add and store per element.)
             const int ldg = R2b + 1;
+            float* Ld = Gs + a.gs_floats - 2 * kRows;          // [row][col mod 2]
             if (r < R2a) {
+                const int dcol = r & ~1;                       // the diagonal block's first column
 #pragma unroll
                 for (int c = 0; c < 64; ++c) {
                     const int col = col0 + c;
-                    if (c < NH && col < R2b) Gs[r * ldg + col] = acc[c] + (use_t ? acc[64 + c] : 0.f);
+                    if (c < NH && col < R2b) {
+                        Gs[r * ldg + col] = use_t ? (col < dcol ? acc[64 + c] : acc[c] + acc[64 + c]) : acc[c];
+                        if (use_t && (col & ~1) == dcol) Ld[2 * r + (col & 1)] = acc[64 + c];
+                    }
                 }
             }
             epi_sync();
-            if (use_t) {
-                // G[col][r] += Dhl[r][col]: each element is touched by one thread here
-                if (r < R2a) {
-#pragma unroll
-                    for (int c = 0; c < 64; ++c) {
-                        const int col = col0 + c;
-                        if (c < NH && col < R2b) Gs[col * ldg + r] += acc[64 + c];
-                    }
-                }
-                epi_sync();
-            }
             const int npl = nb1 * (nb1 + 1) / 2;
             {
                 // kVB pairs per thread at a time: their accumulator loads are
                 // issued together, so their latencies overlap
-                int li = 0;
-                int row_next = nb1;                 // triangle: first index of row li + 1
                 for (int base = et; base < npl; base += kVB * 256) {
                     int pp[kVB];
                     float vre[kVB], vim[kVB];
@@ -729,30 +752,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                         pp[u] = -1;
                         vre[u] = vim[u] = 0.f;
                         if (pl < npl) {
-                            int lj;
-                            if (diag) {
-                                while (pl >= row_next) {
-                                    ++li;
-                                    row_next += nb1 - li;
-                                }
-                                lj = li + (pl - (row_next - (nb1 - li)));
-                            } else {
-                                li = pl / nb2;
-                                lj = pl - li * nb2;
-                            }
+                            const int li = triangle_row(pl, nb1);
+                            const int lj = li + (pl - triangle_start(li, nb1));
                             // block rows 2 i' (Re) and 2 i' + 1 (Im)
-                            const float* g0 = Gs + (2 * li) * ldg + 2 * lj;
-                            const float re = g0[0] + g0[ldg + 1];
-                            const float im = g0[ldg] - g0[1];
-                            const int i = 64 * itm.b1 + li;
-                            const int j = 64 * itm.b2 + lj;
+                            const float* g0 = Gs + 2 * li * ldg + 2 * lj;
+                            float g00 = g0[0], g01 = g0[1], g10 = g0[ldg], g11 = g0[ldg + 1];
+                            if (use_t) {
+                                const bool dg = li == lj;
+                                const float* t = dg ? Ld + 4 * li : Gs + 2 * lj * ldg + 2 * li;
+                                const int st = dg ? 2 : ldg;
+                                g00 += t[0];
+                                g10 += t[1];
+                                g01 += t[st];
+                                g11 += t[st + 1];
+                            }
+                            const float re = g00 + g11;
+                            const float im = g10 - g01;
                             float f;
                             if (MODE == 0)
-                                f = 1.0f / (__ldg(d.split + i) * __ldg(d.split + j));
+                                f = 1.0f / (__ldg(d.split + li) * __ldg(d.split + lj));
                             else
-                                f = 1.0f / (__ldg(d.scale + (int64_t)i * C + itm.k) *
-                                            __ldg(d.scale + (int64_t)j * C + itm.k));
-                            pp[u] = i * N - i * (i - 1) / 2 + (j - i);
+                                f = 1.0f / (__ldg(d.scale + (int64_t)li * C + itm.k) *
+                                            __ldg(d.scale + (int64_t)lj * C + itm.k));
+                            pp[u] = pl;                    // one block: the pair order itself
                             vre[u] = re * f;
                             vim[u] = im * f;
                         }
@@ -760,8 +782,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     if (direct) {
                         double2 old[kVB];
 #pragma unroll
-                        for (int u = 0; u < kVB; ++u)
-                            if (pp[u] >= 0) old[u] = __ldcg(d.acc + (int64_t)itm.k * P + pp[u]);
+                        for (int u = 0; u < kVB; ++u) {
+                            old[u] = make_double2(0.0, 0.0);
+                            if (pp[u] >= 0 && !d.assign) old[u] = __ldcg(d.acc + (int64_t)itm.k * P + pp[u]);
+                        }
 #pragma unroll
                         for (int u = 0; u < kVB; ++u)
                             if (pp[u] >= 0)       // sole owner of (k, p) in this launch
@@ -793,45 +817,63 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     __threadfence();
                     // every pair of the item: the single block's upper
                     // triangle, or a group's nb1 x (64 per B block) rows and
-                    // columns (the diagonal block's upper triangle)
-                    int li = 0;
-                    int row_next = nb1;
+                    // columns (the diagonal block's upper triangle); four pairs
+                    // per thread at a time, their loads in flight together
                     const int npl_all = single ? nb1 * (nb1 + 1) / 2 : nb1 * 64 * itm.nbB;
-                    for (int pl = et; pl < npl_all; pl += 256) {
-                        int i, j;
-                        if (single) {
-                            while (pl >= row_next) {
-                                ++li;
-                                row_next += nb1 - li;
+                    constexpr int kCB = 4;
+                    for (int base = et; base < npl_all; base += kCB * 256) {
+                        int pp[kCB];
+                        double re[kCB], im[kCB];
+#pragma unroll
+                        for (int u = 0; u < kCB; ++u) {
+                            const int pl = base + 256 * u;
+                            pp[u] = -1;
+                            re[u] = im[u] = 0.0;
+                            if (pl >= npl_all) continue;
+                            if (single) {
+                                pp[u] = pl;
+                            } else {
+                                const int i_loc = pl / (64 * itm.nbB);
+                                const int rest = pl - i_loc * 64 * itm.nbB;
+                                const int b2 = itm.b2 + (rest >> 6);
+                                const int j_loc = rest & 63;
+                                if (j_loc >= block_ants(N, b2) || (b2 == itm.b1 && j_loc < i_loc)) continue;
+                                const int i = 64 * itm.b1 + i_loc;
+                                const int j = 64 * b2 + j_loc;
+                                pp[u] = i * N - i * (i - 1) / 2 + (j - i);
                             }
-                            i = li;
-                            j = li + (pl - (row_next - (nb1 - li)));
-                        } else {
-                            const int i_loc = pl / (64 * itm.nbB);
-                            const int rest = pl - i_loc * 64 * itm.nbB;
-                            const int b2 = itm.b2 + (rest >> 6);
-                            const int j_loc = rest & 63;
-                            if (j_loc >= block_ants(N, b2) || (b2 == itm.b1 && j_loc < i_loc)) continue;
-                            i = 64 * itm.b1 + i_loc;
-                            j = 64 * b2 + j_loc;
                         }
-                        const int p = i * N - i * (i - 1) / 2 + (j - i);
-                        double re = 0.0, im = 0.0;
                         for (int sp = 0; sp < pc.nslots; ++sp) {
-                            const float2 v = __ldcg(d.partial + ((int64_t)sp * C + itm.k) * P + p);
-                            re += (double)v.x;
-                            im += (double)v.y;
+                            float2 v[kCB];
+#pragma unroll
+                            for (int u = 0; u < kCB; ++u)
+                                v[u] = pp[u] >= 0 ? __ldcg(d.partial + ((int64_t)sp * C + itm.k) * P + pp[u])
+                                                  : make_float2(0.f, 0.f);
+#pragma unroll
+                            for (int u = 0; u < kCB; ++u) {
+                                re[u] += (double)v[u].x;
+                                im[u] += (double)v[u].y;
+                            }
                         }
                         if (single) {
-                            double2* dst = d.acc + (int64_t)itm.k * P + p;
-                            double2 v = *dst;
-                            v.x += re;
-                            v.y += im;
-                            *dst = v;
+                            double2 old[kCB];
+#pragma unroll
+                            for (int u = 0; u < kCB; ++u) {
+                                old[u] = make_double2(0.0, 0.0);
+                                if (pp[u] >= 0 && !d.assign) old[u] = d.acc[(int64_t)itm.k * P + pp[u]];
+                            }
+#pragma unroll
+                            for (int u = 0; u < kCB; ++u)
+                                if (pp[u] >= 0)
+                                    d.acc[(int64_t)itm.k * P + pp[u]] =
+                                        make_double2(old[u].x + re[u], old[u].y + im[u]);
                         } else {
                             // a group's pass result lives in slot 0 until the
                             // reduction launch adds it to the accumulator
-                            d.partial[(int64_t)itm.k * P + p] = make_float2((float)re, (float)im);
+#pragma unroll
+                            for (int u = 0; u < kCB; ++u)
+                                if (pp[u] >= 0)
+                                    d.partial[(int64_t)itm.k * P + pp[u]] = make_float2((float)re[u], (float)im[u]);
                         }
                     }
                     if (et == 0) d.ticket[itm.k * d.npairs + itm.pr] = 0;
@@ -1006,7 +1048,8 @@ LaunchShape launch_shape(TcPlan* const* plans, int n) {
         L.wide |= plans[m]->nblk > 1;
         if (plans[m]->nblk == 1) r2max = std::max(r2max, 2 * plans[m]->N);
     }
-    L.gs_floats = r2max * (r2max + 1);
+    // G, and in FP32 mode L of its diagonal blocks
+    L.gs_floats = r2max * (r2max + 1) + (plans[0]->mode == 0 ? 2 * kRows : 0);
     L.slot_rows = 8;
     int min_box = kRows;      // the MMA reads 128 rows from a tile: reserve the excess past the ring
     for (int m = 0; m < n; ++m) {
@@ -1244,6 +1287,7 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
         d.ticket = plans[m]->ticket;
         d.scale = runs[m].scale;
         d.split = runs[m].split;
+        d.assign = runs[m].assign;
         d.tiles = d.S_pad / p->KT;
         d.cap_tiles = (int)(p->cap / p->KT);
         d.box_bytes = (uint32_t)p->box_rows * p->row_bytes;
@@ -1257,6 +1301,8 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
         runs[m].n_split = runs[m].direct ? d.n_split : 1;
     }
     a.total_items = base;
+    // (largest dividend of the deal: units x CTAs plus a divisor)
+    a.u32 = (units + 1) * (plans[0]->num_sms + 1) < ((int64_t)1 << 32);
     if (base == 0) return CORR_OK;
     int grid = std::min(base, plans[0]->num_sms);
     if (deal.balanced) {
