@@ -1215,24 +1215,17 @@ int corr_grad(corr_t h, const uint8_t* samples, int64_t n, const float* gains,
 
 namespace {
 
-// The dump kernels of the integration on stream st: the next integration's
-// scales from this one's autocorrelations (when `scales`), then vis[p][k],
-// from the accumulator (which is then cleared) or from a pass result still
-// in partial slot 0 (the accumulator is zero already).
+// The dump of the integration on stream st: vis[p][k], and the next
+// integration's scales from this one's autocorrelations (when `scales`), from
+// the accumulator (which is then cleared) or from a pass result still in
+// partial slot 0 (the accumulator is zero already).
 cudaError_t dump_ops(corr_t h, void* vis, int vis_fp64, bool scales, cudaStream_t st) {
-    cudaError_t e = cudaSuccess;
-    if (h->part_pending) {
-        if (scales)
-            e = launch_scales_from_partial(h->partial, h->N, h->C, h->P, h->n_spec,
-                                           h->scale_target, h->scale, st);
-        if (e == cudaSuccess) e = launch_dump_partial(h->partial, h->C, h->P, vis, vis_fp64, st);
-        h->part_pending = false;
-    } else {
-        if (scales)
-            e = launch_scales_from_autos(h->acc, h->N, h->C, h->P, h->n_spec, h->scale_target,
-                                         h->scale, st);
-        if (e == cudaSuccess) e = launch_dump(h->acc, h->C, h->P, vis, vis_fp64, st);
-    }
+    float* sc = scales ? h->scale : nullptr;
+    const cudaError_t e =
+        h->part_pending
+            ? launch_dump_partial(h->partial, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st)
+            : launch_dump(h->acc, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st);
+    h->part_pending = false;
     h->acc_zero = true;
     return e;
 }

@@ -196,6 +196,6 @@ extern "C" int corr_correlate_noalloc(const uint8_t* samples, int64_t n, int N, 
         if ((e = launch_reduce_partials(part, xa.n_split, (int64_t)C * P, acc, st)) != cudaSuccess)
             return fail_cuda(e, "reduction");
     }
-    if ((e = launch_dump(acc, C, P, vis, 0, st)) != cudaSuccess) return fail_cuda(e, "dump");
+    if ((e = launch_dump(acc, C, P, vis, 0, nullptr, N, 0, 0.0f, st)) != cudaSuccess) return fail_cuda(e, "dump");
     return CORR_OK;
 }

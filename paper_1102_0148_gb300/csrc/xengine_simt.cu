@@ -23,6 +23,7 @@
 // N = 256, K = 1024, 1024 frames 4161 -> 3879, N = 512, K = 64, 2048 frames
 // 3094 -> 2381.
 #include "corr_internal.h"
+#include "scales.cuh"
 
 #include <algorithm>
 
@@ -223,9 +224,18 @@ __device__ __forceinline__ float2 to_f2(float2 v) { return v; }
 __device__ __forceinline__ double2 to_d2(double2 v) { return v; }
 __device__ __forceinline__ double2 to_d2(float2 v) { return make_double2(v.x, v.y); }
 
+// What the dump computes besides vis: the next integration's pre-cast scales
+// from the autocorrelations it passes (scale = nullptr: none).
+struct DumpScales {
+    float* scale;            // [N][C]
+    int N;
+    int64_t n_spec;
+    float target;
+};
+
 template <typename T>
 __global__ void __launch_bounds__(kDT * 8) dump_kernel(const T* __restrict__ acc, int C, int P,
-                                                     void* __restrict__ vis, int fp64) {
+                                                     void* __restrict__ vis, int fp64, DumpScales ds) {
     __shared__ T tile[kDT][kDT + 1];
     const int p0 = blockIdx.x * kDT;
     const int k0 = blockIdx.y * kDT;
@@ -252,6 +262,12 @@ __global__ void __launch_bounds__(kDT * 8) dump_kernel(const T* __restrict__ acc
                 static_cast<double2*>(vis)[e] = to_d2(w);
             else
                 static_cast<float2*>(vis)[e] = to_f2(w);
+            if (ds.scale) {
+                // pair (i, i): the lanes of a warp hold its 32 channels
+                const int i = triangle_row(pp, ds.N);
+                if (triangle_start(i, ds.N) == pp)
+                    ds.scale[(int64_t)i * C + k] = scale_for((double)w.x / (double)ds.n_spec, ds.target);
+            }
         }
     }
 }
@@ -320,18 +336,19 @@ cudaError_t launch_reduce_partials(const float2* partial, int n_split, int64_t C
     return cudaGetLastError();
 }
 
-cudaError_t launch_dump(double2* acc, int C, int P, void* vis, int fp64, cudaStream_t st) {
+cudaError_t launch_dump(double2* acc, int C, int P, void* vis, int fp64, float* scale, int N,
+                        int64_t n_spec, float target, cudaStream_t st) {
     dim3 grid((unsigned)((P + kDT - 1) / kDT), (unsigned)((C + kDT - 1) / kDT));
-    dump_kernel<double2><<<grid, kDT * 8, 0, st>>>(acc, C, P, vis, fp64);
+    dump_kernel<double2><<<grid, kDT * 8, 0, st>>>(acc, C, P, vis, fp64, DumpScales{scale, N, n_spec, target});
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return cudaMemsetAsync(acc, 0, (size_t)C * P * sizeof(double2), st);
 }
 
-cudaError_t launch_dump_partial(const float2* part, int C, int P, void* vis, int fp64,
-                                cudaStream_t st) {
+cudaError_t launch_dump_partial(const float2* part, int C, int P, void* vis, int fp64, float* scale,
+                                int N, int64_t n_spec, float target, cudaStream_t st) {
     dim3 grid((unsigned)((P + kDT - 1) / kDT), (unsigned)((C + kDT - 1) / kDT));
-    dump_kernel<float2><<<grid, kDT * 8, 0, st>>>(part, C, P, vis, fp64);
+    dump_kernel<float2><<<grid, kDT * 8, 0, st>>>(part, C, P, vis, fp64, DumpScales{scale, N, n_spec, target});
     return cudaGetLastError();
 }
 

@@ -45,6 +45,7 @@
 // kernel records a status code, drains its own copies and MMAs, frees TMEM
 // and returns.
 #include "xengine_tc.h"
+#include "scales.cuh"
 #include "tc_ptx.cuh"
 
 #include <cuda.h>
@@ -269,18 +270,6 @@ __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piec
         if (mine) return true;
     }
     return false;
-}
-
-// Upper triangle of n antennas, row-major with autos: first pair of row i, and
-// the row of pair pl.
-__device__ __forceinline__ int triangle_start(int i, int n) { return i * n - i * (i - 1) / 2; }
-__device__ __forceinline__ int triangle_row(int pl, int n) {
-    const float b = 2.0f * n + 1.0f;
-    int i = (int)(0.5f * (b - sqrtf(b * b - 8.0f * pl)));
-    i = min(max(i, 0), n - 1);
-    while (pl < triangle_start(i, n)) --i;             // the root is rounded: at most a step off
-    while (i + 1 < n && pl >= triangle_start(i + 1, n)) ++i;
-    return i;
 }
 
 // Bounded wait with this launch's limit and status word.
