@@ -68,11 +68,14 @@ struct corr_s {
     void* grad_scratch = nullptr; // corr_grad's factor table and partial sums
     float2* partial = nullptr;   // [max_split][C][P]
     int max_split = 0;
-    int* status = nullptr;       // device-side error word
-    // page-locked host memory: the status word's copy, and the corrections as
-    // last uploaded (gains, delays, pre-scales; corr_pin_free follows the
-    // copies that read them)
-    int* status_host = nullptr;
+    // Device-side error word, in page-locked host memory: kernels only write it,
+    // when a wait gives up, and the host reads it after the wait for the stream
+    // without a copy.  The fused kernel, which polls its word, has one on the
+    // device, copied behind its launches.
+    int* status = nullptr;
+    int* fx_status = nullptr;
+    // the corrections as last uploaded (gains, delays, pre-scales), page-locked;
+    // corr_pin_free follows the copies that read them
     float* corr_pin = nullptr;
     cudaEvent_t corr_pin_free = nullptr;
     // host-input staging ring: copies run ahead of the F-engine by up to
@@ -107,7 +110,10 @@ struct corr_s {
     int64_t shifted_frames = 0;
     void* vis_dev = nullptr;
     int64_t n_spec = 0;
-    bool acc_zero = true;        // acc holds zeros (created, or dumped since its last pass)
+    bool acc_zero = true;        // acc counts as zeros (created, or dumped since its last pass)
+    // acc_zero, but the memory still holds the dumped sums: the next pass stores
+    // over them; whatever reads or adds to acc before that clears it (zero_acc)
+    bool acc_stale = false;
     // partial slot 0 holds the integration so far, the pass result of a
     // multi-block mode that went into a zero accumulator, and acc still holds
     // zeros: a dump reads the slot directly, anything else that needs acc or
@@ -212,22 +218,33 @@ int alloc_workspace(corr_t h, int64_t cap) {
     return CORR_OK;
 }
 
-// Queue the copy of the status word behind the handle's work; read_status
-// inspects it once the stream has been waited for.  (One wait for the work and
-// the word: a blocking copy after the wait cost another round trip, ~8 us of a
-// 70 us call.)
+// Queue the fused kernel's status word behind the handle's work (the other
+// kernels' needs no copy); read_status inspects it once the stream has been
+// waited for.
 int queue_status(corr_t h) {
-    CUDA_TRY(h, cudaMemcpyAsync(h->status_host, h->status, sizeof(int), cudaMemcpyDeviceToHost,
-                                h->stream));
+    if (h->fx_status)
+        CUDA_TRY(h, cudaMemcpyAsync(h->status + 1, h->fx_status, sizeof(int), cudaMemcpyDeviceToHost,
+                                    h->stream));
     return CORR_OK;
 }
 
 int read_status(corr_t h) {
-    const int st = *static_cast<volatile int*>(h->status_host);
+    volatile int* s = h->status;
+    const int st = s[0] ? s[0] : s[1];
     if (st != 0) {
-        CUDA_TRY(h, cudaMemset(h->status, 0, sizeof(int)));
+        s[0] = s[1] = 0;
+        if (h->fx_status) CUDA_TRY(h, cudaMemset(h->fx_status, 0, sizeof(int)));
         if (h->tc) tc_reset(h->tc);
         return set_err(h, CORR_ETIMEOUT, "a bounded device-side wait gave up (code %d)", st);
+    }
+    return CORR_OK;
+}
+
+// Clear an accumulator that counts as zeros but still holds dumped sums.
+int zero_acc(corr_t h) {
+    if (h->acc_zero && h->acc_stale) {
+        CUDA_TRY(h, cudaMemsetAsync(h->acc, 0, (size_t)h->C * h->P * sizeof(double2), h->stream));
+        h->acc_stale = false;
     }
     return CORR_OK;
 }
@@ -393,7 +410,7 @@ int fengine_pass(corr_t h, const uint8_t* din, int64_t S, bool raw, int64_t off)
 int settle_partial(corr_t h) {
     if (!h->part_pending) return CORR_OK;
     h->part_pending = false;
-    h->acc_zero = false;
+    h->acc_zero = h->acc_stale = false;
     prof_begin(h);
     CUDA_TRY(h, launch_reduce_partials(h->partial, 1, (int64_t)h->C * h->P, h->acc, h->stream,
                                        true));
@@ -404,7 +421,7 @@ int settle_partial(corr_t h) {
 // FP64 reduction of a tensor-core launch's partials, when it wrote any.
 int finish_tc_run(corr_t h, const TcRun& run, double2* acc) {
     if (run.direct) {           // single-block modes added into acc themselves
-        if (acc == h->acc) h->acc_zero = false;
+        if (acc == h->acc) h->acc_zero = h->acc_stale = false;
         return CORR_OK;
     }
     // a multi-block mode's pass result covers every (k, p) in slot 0: the
@@ -415,7 +432,7 @@ int finish_tc_run(corr_t h, const TcRun& run, double2* acc) {
         return CORR_OK;
     }
     const bool assign = acc == h->acc && h->acc_zero;
-    if (acc == h->acc) h->acc_zero = false;
+    if (acc == h->acc) h->acc_zero = h->acc_stale = false;
     prof_begin(h);
     CUDA_TRY(h, launch_reduce_partials(h->partial, run.n_split, (int64_t)h->C * h->P, acc,
                                        h->stream, assign));
@@ -457,7 +474,7 @@ int xengine_pass(corr_t h, int64_t S_pad, double2* acc) {
         CUDA_TRY(h, launch_xengine_simt(xa, h->stream));
         prof_end(h, CORR_KERNEL_XENGINE);
         const bool assign = acc == h->acc && h->acc_zero;
-        if (acc == h->acc) h->acc_zero = false;
+        if (acc == h->acc) h->acc_zero = h->acc_stale = false;
         prof_begin(h);
         CUDA_TRY(h, launch_reduce_partials(h->partial, xa.n_split, (int64_t)h->C * h->P, acc,
                                            h->stream, assign));
@@ -470,10 +487,11 @@ int xengine_pass(corr_t h, int64_t S_pad, double2* acc) {
 int fx_flush(corr_t h) {
     if (h->fx_pending.empty()) return CORR_OK;
     int src = settle_partial(h);         // the fused kernel adds into acc
+    if (src == CORR_OK) src = zero_acc(h);
     if (src != CORR_OK) return src;
     prof_begin(h);
     int rc = fx_launch(h->fx, h->fx_pending.data(), (int)h->fx_pending.size(), h->twiddle,
-                       split_table(h, false), h->corr_on ? h->corr_tab : nullptr, h->acc, h->status,
+                       split_table(h, false), h->corr_on ? h->corr_tab : nullptr, h->acc, h->fx_status,
                        h->stream, h->err);
     h->acc_zero = false;
     h->fx_pending.clear();
@@ -672,8 +690,8 @@ void destroy_impl(corr_t h) {
     cudaFree(h->acc_raw);
     cudaFree(h->grad_buf);
     cudaFree(h->grad_scratch);
-    cudaFree(h->status);
-    cudaFreeHost(h->status_host);
+    cudaFreeHost(h->status);
+    cudaFree(h->fx_status);
     cudaFreeHost(h->corr_pin);
     if (h->corr_pin_free) cudaEventDestroy(h->corr_pin_free);
     cudaFree(h->vis_dev);
@@ -777,12 +795,12 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
     if (cudaEventCreateWithFlags(&h->f_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->corr_pin_free, cudaEventDisableTiming) != cudaSuccess)
         return bail(set_err(h, CORR_ECUDA, "event creation failed"));
-    if (cudaMallocHost((void**)&h->status_host, sizeof(int)) != cudaSuccess ||
+    if (cudaMallocHost((void**)&h->status, 2 * sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&h->corr_pin, 4 * (size_t)N * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         return bail(set_err(h, CORR_ENOMEM, "host allocation failed"));
     }
-    *h->status_host = 0;
+    h->status[0] = h->status[1] = 0;
     h->f_last = h->stream;
 
     if (h->use_tc) {
@@ -800,7 +818,6 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
     const size_t acc_bytes = (size_t)h->C * h->P * sizeof(double2);
     if (dev_malloc((void**)&h->twiddle, K * sizeof(float2)) != cudaSuccess ||
         dev_malloc((void**)&h->acc, acc_bytes) != cudaSuccess ||
-        dev_malloc((void**)&h->status, sizeof(int)) != cudaSuccess ||
         dev_malloc((void**)&h->corr_tab, (size_t)N * h->C * sizeof(float2)) != cudaSuccess ||
         dev_malloc((void**)&h->gains_dev, (size_t)N * sizeof(float2)) != cudaSuccess ||
         dev_malloc((void**)&h->delays_dev, (size_t)N * sizeof(float)) != cudaSuccess) {
@@ -825,8 +842,7 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
         h->split_host.resize(N);
     }
     if (cudaMemcpy(h->twiddle, tw.data(), K * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemsetAsync(h->acc, 0, acc_bytes, h->stream) != cudaSuccess ||
-        cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) != cudaSuccess)
+        cudaMemsetAsync(h->acc, 0, acc_bytes, h->stream) != cudaSuccess)
         return bail(set_err(h, CORR_ECUDA, "initialisation copy failed"));
     if (h->scale) {
         std::vector<float> ones((size_t)N * h->C, 1.0f);
@@ -887,6 +903,16 @@ int corr_set_fused(corr_t h, int on) {
         if (!fx_supported(h->N, h->K, h->spec_type))
             return set_err(h, CORR_EUNSUPPORTED,
                            "the fused F/X-engine serves K = 512, CORR_FP32, N <= %d", kFxMaxN);
+        if (!h->fx_status) {
+            int* s = nullptr;
+            CUDA_TRY(h, dev_malloc((void**)&s, sizeof(int)));
+            if (cudaMemset(s, 0, sizeof(int)) != cudaSuccess) {
+                cudaGetLastError();
+                cudaFree(s);
+                return set_err(h, CORR_ECUDA, "initialisation failed");
+            }
+            h->fx_status = s;
+        }
         std::string ferr;
         const int rc = fx_plan_create(&h->fx, h->N, ferr);
         if (rc != CORR_OK) return set_err(h, rc, "%s", ferr.c_str());
@@ -975,6 +1001,7 @@ int corr_save_state(corr_t h, void* buf) {
     if (!h || !buf) return CORR_EINVAL;
     int frc = flush(h);
     if (frc == CORR_OK) frc = settle_partial(h);
+    if (frc == CORR_OK) frc = zero_acc(h);
     if (frc != CORR_OK) return frc;
     int rc = wait_and_check(h);
     if (rc != CORR_OK) return rc;
@@ -1013,7 +1040,7 @@ int corr_load_state(corr_t h, const void* buf) {
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     const unsigned char* p = static_cast<const unsigned char*>(buf) + sizeof hd;
     const size_t ab = (size_t)h->C * h->P * sizeof(double2);
-    h->acc_zero = false;
+    h->acc_zero = h->acc_stale = false;
     h->part_pending = false;
     CUDA_TRY(h, cudaMemcpy(h->acc, p, ab, cudaMemcpyHostToDevice));
     p += ab;
@@ -1217,14 +1244,23 @@ namespace {
 
 // The dump of the integration on stream st: vis[p][k], and the next
 // integration's scales from this one's autocorrelations (when `scales`), from
-// the accumulator (which is then cleared) or from a pass result still in
-// partial slot 0 (the accumulator is zero already).
-cudaError_t dump_ops(corr_t h, void* vis, int vis_fp64, bool scales, cudaStream_t st) {
+// the accumulator or from a pass result still in partial slot 0 (the
+// accumulator counts as zero already).  The dumped accumulator is not cleared:
+// the next pass stores over it.  A dump of no pass at all clears it first;
+// `recording` (a graph, whose replays follow any eager use) does so whatever
+// the memory holds now.
+cudaError_t dump_ops(corr_t h, void* vis, int vis_fp64, bool scales, cudaStream_t st, bool recording) {
     float* sc = scales ? h->scale : nullptr;
-    const cudaError_t e =
-        h->part_pending
-            ? launch_dump_partial(h->partial, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st)
-            : launch_dump(h->acc, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st);
+    cudaError_t e = cudaSuccess;
+    if (h->part_pending) {
+        e = launch_dump_partial(h->partial, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st);
+    } else {
+        if (h->acc_zero && (h->acc_stale || recording))
+            e = cudaMemsetAsync(h->acc, 0, (size_t)h->C * h->P * sizeof(double2), st);
+        if (e == cudaSuccess)
+            e = launch_dump(h->acc, h->C, h->P, vis, vis_fp64, sc, h->N, h->n_spec, h->scale_target, st);
+        h->acc_stale = !h->acc_zero || recording;
+    }
     h->part_pending = false;
     h->acc_zero = true;
     return e;
@@ -1243,7 +1279,7 @@ int enqueue_dump(corr_t h, void* vis, int vis_fp64, bool dev) {
     // the next integration is scaled from this one's autocorrelations
     const bool scales = narrow(h) && !h->scales_user && h->n_spec > 0;
     prof_begin(h);
-    CUDA_TRY(h, dump_ops(h, out, vis_fp64, scales, h->stream));
+    CUDA_TRY(h, dump_ops(h, out, vis_fp64, scales, h->stream, false));
     if (scales) h->scales_ready = true;
     prof_end(h, CORR_KERNEL_DUMP);
     if (!dev) CUDA_TRY(h, cudaMemcpyAsync(vis, out, bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1634,7 +1670,7 @@ int corr_batch_capture(corr_batch_t b, const uint8_t* const* samples, const int6
         rc = batch_enqueue(b, samples, n);
         for (int m = 0; rc == CORR_OK && m < b->n; ++m) {
             corr_t h = b->h[m];
-            e = dump_ops(h, vis[m], vis_fp64, narrow(h) && !h->scales_user, b->stream);
+            e = dump_ops(h, vis[m], vis_fp64, narrow(h) && !h->scales_user, b->stream, true);
             if (e != cudaSuccess) rc = CORR_ECUDA;
         }
         cudaGraph_t g = nullptr;

@@ -146,13 +146,12 @@ cudaError_t launch_xengine_simt(XengineArgs& a, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float2* partial, int n_split, int64_t CP,
                                    double2* acc, cudaStream_t st, bool assign = false);
 
-// vis[p][k] = acc[k][p] as complex64 (fp64 == 0) or complex128; then acc = 0.
+// vis[p][k] = acc[k][p] as complex64 (fp64 == 0) or complex128.
 // scale != nullptr: also the pre-cast scales of the next integration from the
 // autocorrelations over n_spec spectra ([N][C], see scales.cuh).
-cudaError_t launch_dump(double2* acc, int C, int P, void* vis, int fp64, float* scale, int N,
+cudaError_t launch_dump(const double2* acc, int C, int P, void* vis, int fp64, float* scale, int N,
                         int64_t n_spec, float target, cudaStream_t st);
-// The same from a pass result still in partial slot 0 (part[k][p], FP32),
-// with the accumulator already zero: nothing is cleared.
+// The same from a pass result still in partial slot 0 (part[k][p], FP32).
 cudaError_t launch_dump_partial(const float2* part, int C, int P, void* vis, int fp64, float* scale,
                                 int N, int64_t n_spec, float target, cudaStream_t st);
 

@@ -160,9 +160,12 @@ extern "C" int corr_correlate_noalloc(const uint8_t* samples, int64_t n, int N, 
                                            max_split * part_bytes);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-    // The array keeps the previous call's contents: clear the accumulator.
-    e = cudaMemsetAsync(acc, 0, (size_t)C * P * sizeof(double2), st);
-    if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
+    // The array keeps the previous call's contents: the first pass stores over
+    // the accumulator, and a call without a pass clears it.
+    if (n == 0) {
+        e = cudaMemsetAsync(acc, 0, (size_t)C * P * sizeof(double2), st);
+        if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
+    }
     noalloc_twiddles<<<(K + 255) / 256, 256, 0, st>>>(tw, K);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e, "twiddle kernel");
 
@@ -193,7 +196,7 @@ extern "C" int corr_correlate_noalloc(const uint8_t* samples, int64_t n, int N, 
         xa.max_split = max_split;
         xa.partial = part;
         if ((e = launch_xengine_simt(xa, st)) != cudaSuccess) return fail_cuda(e, "X-engine");
-        if ((e = launch_reduce_partials(part, xa.n_split, (int64_t)C * P, acc, st)) != cudaSuccess)
+        if ((e = launch_reduce_partials(part, xa.n_split, (int64_t)C * P, acc, st, f0 == 0)) != cudaSuccess)
             return fail_cuda(e, "reduction");
     }
     if ((e = launch_dump(acc, C, P, vis, 0, nullptr, N, 0, 0.0f, st)) != cudaSuccess) return fail_cuda(e, "dump");

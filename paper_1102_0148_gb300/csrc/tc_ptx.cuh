@@ -67,7 +67,8 @@ __device__ __forceinline__ bool wait_bar_t(uint32_t bar, uint32_t parity, volati
                 t0 = now;
             } else if (now - t0 > timeout_ns) {
                 *abort_word = 1;
-                atomicCAS(status, 0, kStatusTimeout);
+                *static_cast<volatile int*>(status) = kStatusTimeout;   // may be host memory
+                __threadfence_system();
                 return false;
             }
         }

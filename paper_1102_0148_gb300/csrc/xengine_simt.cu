@@ -211,9 +211,8 @@ __global__ void reduce_partials_kernel(const float2* part, int n_split, int64_t 
 }
 
 // acc [C][P] -> vis [P][C] through 32 x 32 shared-memory tiles, so both the
-// reads (along p) and the writes (along k) are coalesced.  (acc is cleared by
-// a memset after it: zero stores here, to the lines just loaded, held the
-// kernel to a quarter of the HBM bandwidth.)  T = double2 for the FP64
+// reads (along p) and the writes (along k) are coalesced.  (acc keeps its
+// sums: the next pass stores over them.)  T = double2 for the FP64
 // accumulator, float2 for a pass result still in partial slot 0 (its FP64
 // reduction into a zero accumulator would give the same values); values
 // change type only on the way out, as FP64 conversions are slow here.
@@ -336,13 +335,11 @@ cudaError_t launch_reduce_partials(const float2* partial, int n_split, int64_t C
     return cudaGetLastError();
 }
 
-cudaError_t launch_dump(double2* acc, int C, int P, void* vis, int fp64, float* scale, int N,
+cudaError_t launch_dump(const double2* acc, int C, int P, void* vis, int fp64, float* scale, int N,
                         int64_t n_spec, float target, cudaStream_t st) {
     dim3 grid((unsigned)((P + kDT - 1) / kDT), (unsigned)((C + kDT - 1) / kDT));
     dump_kernel<double2><<<grid, kDT * 8, 0, st>>>(acc, C, P, vis, fp64, DumpScales{scale, N, n_spec, target});
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return cudaMemsetAsync(acc, 0, (size_t)C * P * sizeof(double2), st);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_dump_partial(const float2* part, int C, int P, void* vis, int fp64, float* scale,
