@@ -375,23 +375,23 @@ __global__ void __launch_bounds__(kFxThreads, 1) fx_fused_kernel(const __grid_co
                                 const uint32_t ab = base + (uint32_t)at * L.atom;
 #pragma unroll
                                 for (int kk = 0; kk < 2; ++kk) {
-                                    const uint64_t ah = sw64_desc(ab + 32u * kk);
-                                    const uint64_t al = sw64_desc(ab + L.slot + 32u * kk);
-                                    mma<0>(tmem, ah, ah, idesc, accum);
-                                    mma<0>(tmem, al, ah, idesc_lh, 1u);
+                                    const uint64_t ah = op_desc<0>(op_desc_lo(ab + 32u * kk));
+                                    const uint64_t al = op_desc<0>(op_desc_lo(ab + L.slot + 32u * kk));
+                                    mma<0, 1>(tmem, ah, ah, idesc, accum);
+                                    mma<0, 1>(tmem, al, ah, idesc_lh, 1u);
                                     accum = 1;
                                 }
                             }
                             issued = true;
-                            mma_commit(smem_u32(&empty[st]));
+                            mma_commit<1>(smem_u32(&empty[st]));
                         }
                         if (!ok) break;
-                        mma_commit(smem_u32(accf));
+                        mma_commit<1>(smem_u32(accf));
                     }
                 }
             }
             if (!ok && issued) {
-                mma_commit(smem_u32(drain));
+                mma_commit<1>(smem_u32(drain));
                 const unsigned long long d2 = globaltimer() + a.timeout_ns;
                 while (!mbar_try_wait(smem_u32(drain), 0u))
                     if (globaltimer() > d2) break;

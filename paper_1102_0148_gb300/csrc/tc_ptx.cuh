@@ -51,6 +51,33 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Arrive at the barrier at this shared-memory offset in CTA `rank` of the
+// cluster.
+__device__ __forceinline__ void mbar_arrive_rank(uint32_t bar, uint32_t rank) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\t"
+        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
+        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar),
+        "r"(rank)
+        : "memory");
+}
+
+// The same with nothing of this thread's own to release: it passes on the
+// completion of TMA copies, which have landed.  (With .release.cluster, a
+// fence per stage, an FP16 pass at N = 256 took 716 us, not 589.)
+__device__ __forceinline__ void mbar_relay(uint32_t bar, uint32_t rank) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\t"
+        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
+        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar),
+        "r"(rank)
+        : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Bounded wait on phase `parity` of `bar`.  Returns false on timeout or when
 // another role has already given up (the shared abort word is set); on
 // timeout it sets the abort word and records kStatusTimeout in `status`.
@@ -93,56 +120,69 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
-// 1024 bytes apart, descriptor version 1 (bits 46-47), layout type 2 (bits 61-63).
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
-// The same for 64-byte rows: 64-byte swizzle, 8-row groups 512 bytes apart,
-// layout type 4.
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(512u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
-
-// Operand descriptor of a tile row layout: FP16 modes 64-byte rows, FP8 128.
-template <int MODE>
-__device__ __forceinline__ uint64_t op_desc(uint32_t saddr) {
-    return MODE == 2 ? sw128_desc(saddr) : sw64_desc(saddr);
-}
+// Shared-memory matrix descriptor of a K-major tile row layout, low word:
+// start address and the (unused) leading offset in 16-byte units; adding to
+// it moves the start.  High word: 8-row groups 512 bytes apart and the 64-byte
+// swizzle (layout type 4 at bits 61-63) for 64-byte rows (FP16 modes), 1024
+// and the 128-byte swizzle (2) for 128-byte rows (FP8); descriptor version 1
+// at bits 46-47.
+__device__ __forceinline__ uint32_t op_desc_lo(uint32_t saddr) { return (saddr & 0x3FFFFu) >> 4 | 1u << 16; }
 
 template <int MODE>
+__device__ __forceinline__ uint64_t op_desc(uint32_t lo) {
+    constexpr uint32_t hi = MODE == 2 ? 1024u >> 4 | 1u << 14 | 2u << 29 : 512u >> 4 | 1u << 14 | 4u << 29;
+    return (uint64_t)hi << 32 | lo;
+}
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// CG: CTAs that share the MMA (cta_group::1 or ::2, issued by rank 0 of the
+// pair; the descriptors hold in both CTAs).
+template <int MODE, int CG>
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                     uint32_t accumulate) {
+#define GBCORR_MMA(group, kind)                                                          \
+    asm volatile(                                                                        \
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"                                \
+        "tcgen05.mma.cta_group::" group ".kind::" kind " [%0], %1, %2, %3, p;\n\t}" ::"r"( \
+            d_tmem),                                                                     \
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)                              \
+        : "memory")
     if (MODE == 2) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
+        if (CG == 1)
+            GBCORR_MMA("1", "f8f6f4");
+        else
+            GBCORR_MMA("2", "f8f6f4");
     } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
+        if (CG == 1)
+            GBCORR_MMA("1", "f16");
+        else
+            GBCORR_MMA("2", "f16");
     }
+#undef GBCORR_MMA
 }
 
+// Arrives at the barrier (CG 2: at this offset in both CTAs of the pair) once
+// the MMAs issued so far are done.
+template <int CG>
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
+    if (CG == 1)
+        asm volatile(
+            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+            " [%0], %1;" ::"r"(bar),
+            "h"((uint16_t)3)
+            : "memory");
 }
 
 __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, uint32_t src, int c0, int c1,

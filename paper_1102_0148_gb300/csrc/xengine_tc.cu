@@ -13,7 +13,8 @@
 //   Re V_ij = G[2i'][2j'] + G[2i'+1][2j'+1],  Im V_ij = G[2i'+1][2j'] - G[2i'][2j'+1].)
 // Each block pair is a dense contraction D[128 x Nn] += A_b1[128 x 16|32] *
 // A_b2^T on the tensor cores, operands loaded by TMA (rows past the antenna
-// count are zero-filled), FP32 accumulators in TMEM.  For a diagonal pair
+// count are zero-filled), FP32 accumulators in TMEM.  With several blocks a
+// pair of CTAs takes two blocks against two at a time.  For a diagonal pair
 // both operands are the same shared-memory tile.
 //
 // Precisions (operands in shared memory, K-major; FP16 tiles of 32 spectra in
@@ -29,13 +30,19 @@
 //   mode 2: one FP8-E4M3 plane (pre-scaled), kind::f8f6f4.
 //
 // One launch may serve several correlators ("modes") of different N and K
-// that share the precision: work items (mode, channel, block pair, range of
-// spectra) are enumerated mode by mode and dealt round-robin to persistent
-// CTAs of 10 warps:
-//   warp 0    TMA producer (one lane)     -> stage ring (full/empty mbarriers)
-//   warp 1    TMEM allocator + MMA issuer (one lane) -> two TMEM accumulator sets
+// that share the precision: work items (mode, channel, block pair or group,
+// range of spectra) are enumerated mode by mode and dealt round-robin to
+// persistent CTAs (several blocks: CTA pairs) of 10 warps:
+//   warp 0    TMA producer                -> stage ring (full/empty mbarriers)
+//   warp 1    TMEM allocator + MMA issuer -> two TMEM accumulator sets
 //   warps 2-9 epilogue: TMEM -> registers, summed over windows -> G in shared
 //             memory -> V -> FP64 accumulator (or FP32 partials)
+// What the MMA warp does per stage sets the pace, not the tensor pipe: a loop
+// of one lane spent ~1500 clocks on a stage of 8 MMAs (128 clocks each),
+// ~100 an MMA, on descriptors built for each and copied to uniform registers,
+// and ~130 a wait.  Now the warp runs whole, one elected lane issues, and a
+// descriptor is the stage's plus a constant: 130 antennas, K = 2048, 1500
+// spectra FP16 418 -> 352 us, N = 11, K = 4096, 1024 spectra 94 -> 63 us.
 // The tensor core's FP32 accumulation into TMEM is biased (it loses about one
 // unit in the last place per accumulate, always toward zero), so TMEM only
 // accumulates one window of W spectra; the epilogue adds the windows with
@@ -79,7 +86,7 @@ struct TcModeArgs {
     int64_t unit_base;        // first work unit of this mode (balanced deal)
     float2* partial;          // [n_split][C][P] FP32 partials (n_split > 1)
     double2* acc;             // [C][P] FP64 accumulator
-    int* ticket;              // [C][npairs] arrival counters (n_split > 1), zero between launches
+    int* ticket;              // [C][npairs][CTAs of a worker] arrival counters (n_split > 1), zero between launches
     const float* scale;       // [N][C] pre-cast scales (modes 1, 2)
     const float* split;       // [N] two-plane pre-scales sigma_i (mode 0)
     int assign;               // acc is known to hold zeros: store instead of adding
@@ -93,7 +100,7 @@ struct TcArgs {
     int kt_shift;             // log2(KT): the single-lane roles avoid 64-bit division
     int atoms;                // k-tiles of KT spectra per pipeline stage
     int row_bytes;            // bytes of one tile row: 64 (FP16 modes) or 128 (FP8)
-    int wide;                 // a mode has several antenna blocks: atoms hold A, B0, B1 slots
+    int wide;                 // modes of several antenna blocks: atoms hold A and B slots
     int gs_floats;            // epilogue G buffer (largest 2nb x (2nb + 1) of the modes; FP32 mode + 2 kRows)
     int slot_rows;            // rows of one operand tile slot in shared memory (<= 128)
     int* status;
@@ -117,31 +124,37 @@ struct Piece {
 };
 
 // Work groups of a channel.  One antenna block (N <= 64): the single
-// diagonal block pair.  Several blocks: block b1 against the blocks
-// b2 .. b2 + nbB - 1 (b2 = b1, b1 + 2, ...; nbB = 2, or 1 for the last one of
-// a row), so one A tile feeds an MMA of N = 256 and a channel's 4 blocks
-// (N = 256 antennas) take 6 groups instead of 10 pairs.
+// diagonal block pair.  Several blocks: two blocks (b1, b1 + 1; the A rows of
+// the two CTAs of a pair) against two blocks (b2, b2 + 1; half of the B rows
+// in each CTA), b1 <= b2, both even: 4 blocks (N = 256 antennas) take 3
+// groups.  nbB is the number of B blocks that exist.
 __host__ __device__ __forceinline__ int groups_of(int nblk) {
-    if (nblk == 1) return 1;
-    int g = 0;
-    for (int b1 = 0; b1 < nblk; ++b1) g += (nblk - b1 + 1) >> 1;
-    return g;
+    const int nb2 = (nblk + 1) >> 1;
+    return nb2 * (nb2 + 1) / 2;
 }
 
 __host__ __device__ __forceinline__ void group_decode(int gi, int nblk, int& b1, int& b2, int& nbB) {
-    b1 = 0;
-    if (nblk > 1)
-        while (gi >= ((nblk - b1 + 1) >> 1)) {
-            gi -= (nblk - b1 + 1) >> 1;
-            ++b1;
-        }
-    b2 = b1 + 2 * gi;
-    nbB = nblk == 1 ? 1 : (nblk - b2 < 2 ? nblk - b2 : 2);
+    const int nb2 = (nblk + 1) >> 1;
+    int r = 0;
+    while (gi >= nb2 - r) {
+        gi -= nb2 - r;
+        ++r;
+    }
+    b1 = 2 * r;
+    b2 = 2 * (r + gi);
+    nbB = nblk - b2 < 2 ? nblk - b2 : 2;
+}
+
+// Columns of a group: its B rows, rounded up to 64 (half of them in each CTA
+// and in each half of the epilogue's warps, in whole 16-baseline rounds).
+__host__ __device__ __forceinline__ int group_cols(int N, int b2) {
+    const int c = (2 * N - 128 * b2 + 63) & ~63;
+    return c < 256 ? c : 256;
 }
 
 // Work units per k-tile: 2 for the single diagonal pair (one tile loaded,
-// two MMAs in FP32 mode); for a group, one per tile loaded (an A tile that
-// is the group's first B block is not loaded again) plus one.  Each item
+// two MMAs in FP32 mode); for a group, one per tile that a CTA loads (on the
+// diagonal its A tile is also its half of B) plus one.  Each item
 // (with k-tiles) starts with kEndUnits more, standing for the cost of an
 // item's end (~4 k-tiles); they hold no k-tile.
 constexpr int kEndUnits = 8;
@@ -153,10 +166,17 @@ __host__ __device__ __forceinline__ int pair_units(int gi, int nblk) {
     if (nblk == 1) return 2;
     int b1, b2, nbB;
     group_decode(gi, nblk, b1, b2, nbB);
-    return nbB + (b2 != b1 ? 1 : 0) + 1;
+    return b2 != b1 ? 3 : 2;
 }
 
-__device__ __forceinline__ Item decode_item(const TcArgs& a, int g) {
+// How far the groups of the channel whose first item is g0 are turned.
+__host__ __device__ __forceinline__ int group_turn(int g0, int npairs, int G) {
+    const int step = (npairs + 1 - G % npairs) % npairs;
+    return (int)((int64_t)step * (g0 / G) % npairs);
+}
+
+// Item g of the round-robin deal to G workers.
+__device__ __forceinline__ Item decode_item(const TcArgs& a, int g, int G) {
     int m = 0;
     while (m + 1 < a.n_modes && g >= a.md[m + 1].item_base) ++m;
     const TcModeArgs& d = a.md[m];
@@ -164,9 +184,14 @@ __device__ __forceinline__ Item decode_item(const TcArgs& a, int g) {
     Item it;
     it.m = m;
     // group fastest: the CTAs that take one channel's groups at the same
-    // time share its block tiles through L2
-    const int pr = l % d.npairs;
+    // time share its block tiles through L2.  The order of a channel's groups
+    // is turned by one deal round after another so that a worker's group
+    // index steps by one per round, whatever G is modulo npairs: groups cost
+    // 2 or 3 units, and with G a multiple of npairs a worker would only ever
+    // see one of them
+    int pr = l % d.npairs;
     l /= d.npairs;
+    if (d.npairs > 1) pr = (pr + group_turn(d.item_base + l * d.npairs, d.npairs, G)) % d.npairs;
     it.pr = pr;
     it.k = l % d.C;
     it.sp = l / d.C;
@@ -200,10 +225,11 @@ __device__ __forceinline__ int64_t ceil_div(const TcArgs& a, int64_t x, int64_t 
     return deal_div(a, x + y - 1, y);
 }
 
+template <bool WIDE>
 __device__ __forceinline__ void cursor_init(const TcArgs& a, PieceCursor& c) {
-    c.g = blockIdx.x;
+    c.g = WIDE ? blockIdx.x >> 1 : blockIdx.x;
     c.m = a.n_modes;
-    if (!a.balanced) return;
+    if (WIDE || !a.balanced) return;
     const int64_t G = gridDim.x;
     c.lo = ceil_div(a, (int64_t)blockIdx.x * a.units, G);
     c.hi = ceil_div(a, (int64_t)(blockIdx.x + 1) * a.units, G);
@@ -225,16 +251,18 @@ __device__ __forceinline__ void cursor_init(const TcArgs& a, PieceCursor& c) {
     }
 }
 
+template <bool WIDE>
 __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piece& p) {
-    if (!a.balanced) {
+    if (WIDE || !a.balanced) {
         if (c.g >= a.total_items) return false;
-        p.itm = decode_item(a, c.g);
+        const int G = WIDE ? gridDim.x >> 1 : gridDim.x;      // workers: CTA pairs or CTAs
+        p.itm = decode_item(a, c.g, G);
         const TcModeArgs& d = a.md[p.itm.m];
         p.s_beg = (int64_t)p.itm.sp * d.S_item;
         p.s_end = min(d.S_pad, p.s_beg + d.S_item);
         p.slot = p.itm.sp;
         p.nslots = d.n_split;
-        c.g += gridDim.x;
+        c.g += G;
         return true;
     }
     const int64_t G = gridDim.x;
@@ -283,24 +311,22 @@ __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" :::
 
 // --------------------------------------------------------------------- kernel
 
-// Stage layout of one item.  A group (several antenna blocks) fills each
-// k-tile's atom of the launch's layout.  A single-block item packs its tiles
-// densely: atom = [hi | lo] tiles of its own box (2N rows rounded up to 8),
-// as many per stage as fit and divide a window, so a single-block mode in a
-// launch with a multi-block one still moves up to a window of spectra per
-// stage handshake.  (In a launch of single-block modes only this is the
-// launch's own layout for the largest mode and denser for smaller ones.)
+// Stage layout of one item.  A group with its own B slots fills each k-tile's
+// atom of the launch's layout.  An item whose A tiles are also its B tiles
+// (single block, group on the diagonal) packs them densely: atom = [hi | lo]
+// tiles of its mode's box (one block: 2N rows rounded up to 8), as many per
+// stage as fit and divide a window.
 struct ItemLayout {
     uint32_t atom;      // bytes per k-tile
     uint32_t plo;       // hi -> lo plane within a k-tile
     int at;             // k-tiles per stage
 };
 
-__device__ __forceinline__ ItemLayout item_layout(const TcArgs& a, const TcModeArgs& d, bool single,
+__device__ __forceinline__ ItemLayout item_layout(const TcArgs& a, const TcModeArgs& d, bool dense,
                                                   int planes, uint32_t stage_bytes,
                                                   uint32_t atom_bytes, uint32_t plane_off) {
     ItemLayout L;
-    if (!single) {
+    if (!dense) {
         L.atom = atom_bytes;
         L.plo = plane_off;
         L.at = a.atoms;
@@ -315,20 +341,30 @@ __device__ __forceinline__ ItemLayout item_layout(const TcArgs& a, const TcModeA
     return L;
 }
 
-// WIDE: some mode of the launch has several antenna blocks (work groups of
-// one A block and two B blocks); launches of single-block modes only take
-// the narrow instance, which has none of the group code.
+// WIDE: modes of several antenna blocks, worked on by pairs of CTAs (clusters
+// of two, tcgen05 cta_group::2).  A pair's MMA is M = 256 (each CTA's 128 A
+// rows, one antenna block), N up to 256 (half of the B rows in each CTA's
+// shared memory); each CTA's TMEM holds its own 128 rows.  A CTA reads 8 KB
+// of operands per K = 16 step of 128 clocks, the shared-memory rate at which
+// MMAs are fed (~64 bytes per clock: alone, a CTA's 128 x 256 tile reads 12
+// KB per step and ran at 60% of the tensor rate with its loads taken away),
+// and loads 8 tiles per channel and k-tile at N = 256, not 12.  A pass of
+// 4096 spectra at N = 256, K = 1024: FP32 mode 2033 -> 1393 us, FP16 831 ->
+// 530, FP8 371 -> 275 (with the scales and the issue loop below).
+// Rank 0 issues the MMAs: its own tiles' barrier and the other CTA's, whose
+// warp 1 passes each full stage on by a remote arrival.  Commits arrive at
+// both CTAs' barriers; the epilogue warps of both free an accumulator set.
+// Each CTA loads with its own TMA into its own barriers, so each can wait for
+// its own copies if the launch gives up.
 template <int MODE, bool WIDE>
 __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_constant__ TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int planes = MODE == 0 ? 2 : 1;
-    // Stage layout of a group (several antenna blocks, WIDE): per k-tile
-    // ("atom") the A slot of each plane [hi | lo], then the B slots
-    // [B0 hi | B1 hi | B0 lo | B1 lo] (one plane: [B0 | B1]), so a group's
-    // two B blocks form one operand of 256 rows; a slot has slot_rows = 128
-    // rows.  A single-block item packs its k-tiles densely instead
+    // Stage layout of a group (WIDE): per k-tile ("atom") the A slot of each
+    // plane [hi | lo], then the B half's; a slot has slot_rows = 128 rows.  A
+    // single-block item packs its k-tiles densely instead
     // ([hi | lo] of its own 2N-rounded-up-to-8 rows each, item_layout).  The
     // MMA reads 128 rows from a tile (and a single block's concatenated
     // [hi; lo] B operand 2 box rows); rows past the antennas only feed
@@ -337,12 +373,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
     const uint32_t slot = (uint32_t)a.slot_rows * (uint32_t)a.row_bytes;
     constexpr int KK = MODE == 2 ? 4 : 2;       // MMA k-steps (32 bytes of a row) per k-tile
     const uint32_t plane_off = slot;                                // A: hi -> lo plane
-    const uint32_t bh_off = planes * slot;                          // B0 hi (B1 hi follows)
-    const uint32_t bl_off = bh_off + 2 * slot;                      // B0 lo (planes == 2)
-    const uint32_t atom_bytes = planes * slot * (WIDE ? 3u : 1u);
+    const uint32_t bh_off = planes * slot;                          // B half: hi
+    const uint32_t bl_off = bh_off + slot;                          // B half: lo (planes == 2)
+    const uint32_t atom_bytes = planes * slot * (WIDE ? 2u : 1u);
+    constexpr bool single = !WIDE;
+    const int rank = WIDE ? (int)(blockIdx.x & 1) : 0;              // CTA of the pair
     const uint32_t stage_bytes = atom_bytes * (uint32_t)a.atoms;
     unsigned char* stages = smem;
-    float* Gs = reinterpret_cast<float*>(smem + a.stages * stage_bytes);   // <= 128 x 129
+    float* Gs = reinterpret_cast<float*>(smem + a.stages * stage_bytes);   // <= 128 x 129; WIDE: scales
     // WIDE: each epilogue warp's staging rows for V, [16][kVRow] float2
     float2* vstage = reinterpret_cast<float2*>(Gs + a.gs_floats);
     uint64_t* bars = reinterpret_cast<uint64_t*>(
@@ -366,12 +404,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < a.stages; ++s) {
-            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&full[s]), WIDE && rank == 0 ? 2 : 1);   // own copies, relay
             mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&accf[b]), 1);
-            mbar_init(smem_u32(&acce[b]), 8);      // one arrival per epilogue warp
+            mbar_init(smem_u32(&acce[b]), WIDE ? 16 : 8);      // one arrival per epilogue warp
         }
         mbar_init(smem_u32(drain), 1);
         *abort_word = 0;
@@ -379,177 +417,221 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(tmem_slot)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (WIDE) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(tmem_slot)),
+                         "r"(kTmemCols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(tmem_slot)),
+                         "r"(kTmemCols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
-    __syncthreads();
+    if (WIDE)
+        cluster_sync();
+    else
+        __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         // ------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            uint32_t it = 0, st = 0, ph = 0;       // stage slot and its phase parity
-            uint32_t armed = 0, armed_ph = 0;     // slots with copies in flight, their parity
-            bool ok = true;
-            PieceCursor cur;
-            cursor_init(a, cur);
-            Piece pc;
-            while (ok && next_piece(a, cur, pc)) {
-                const Item& itm = pc.itm;
-                const TcModeArgs& d = a.md[itm.m];
-                const CUtensorMap* map = &a.tmap[itm.m];
-                const bool single = !WIDE || d.nblk == 1;  // one block: A = B, one tile
-                const bool alias = !single && itm.b2 == itm.b1;   // A is the group's first B block
-                const int ra = kRows * itm.b1;
-                const int rb = kRows * itm.b2;
-                const uint32_t ntile = single ? 1u : (uint32_t)itm.nbB + (alias ? 0u : 1u);
-                const ItemLayout lay = item_layout(a, d, single, planes, stage_bytes, atom_bytes, plane_off);
-                const int step_i = a.KT * lay.at;
-                const int64_t s_beg = pc.s_beg;
-                const int64_t s_end = pc.s_end;
-                for (int64_t s = s_beg; s < s_end; s += step_i, ++it) {
-                    if (it > 0 && ++st == (uint32_t)a.stages) {
-                        st = 0;
-                        ph ^= 1u;
-                    }
-                    if (!wait_bar(smem_u32(&empty[st]), ph ^ 1u, abort_word, a)) {
-                        ok = false;
-                        break;
-                    }
-                    if (a.withhold && blockIdx.x == 0 && it == 0) continue;   // test hook
-                    const int n_at = (int)min((int64_t)lay.at, (s_end - s) >> a.kt_shift);
-                    const uint32_t bytes = (uint32_t)n_at * planes * d.box_bytes * ntile;
+        // (Warps 0 and 1 run their loops whole, with one elected lane issuing:
+        // addresses and descriptors then live in uniform registers, which a
+        // loop of one lane has to fill again for every instruction.)
+        const bool el = elect_one();
+        uint32_t st = 0, ph = 0;               // stage slot and its phase parity
+        uint32_t armed = 0, armed_ph = 0;      // slots with copies in flight, their parity
+        bool ok = true, first = true;
+        const uint32_t stage0 = smem_u32(stages);
+        PieceCursor cur;
+        cursor_init<WIDE>(a, cur);
+        Piece pc;
+        while (ok && next_piece<WIDE>(a, cur, pc)) {
+            const Item& itm = pc.itm;
+            const TcModeArgs& d = a.md[itm.m];
+            const CUtensorMap* map = &a.tmap[itm.m];
+            // one block: A = B, one tile.  Group on the diagonal: A is the
+            // CTA's half of B (if both blocks are there)
+            const int cols = group_cols(d.N, itm.b2);
+            const bool alias = single || (itm.b2 == itm.b1 && cols == 256);
+            const int ra = kRows * (itm.b1 + rank);
+            const int rb = kRows * itm.b2 + rank * (cols >> 1);
+            const uint32_t tile_bytes = planes * d.box_bytes * (alias ? 1u : 2u);
+            const ItemLayout lay = item_layout(a, d, alias, planes, stage_bytes, atom_bytes, plane_off);
+            const int t_end = (int)(pc.s_end >> a.kt_shift);
+            for (int t = (int)(pc.s_beg >> a.kt_shift); t < t_end; t += lay.at) {
+                if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&empty[st]), ph ^ 1u, abort_word, a))) {
+                    ok = false;
+                    break;
+                }
+                if (!(a.withhold && blockIdx.x == 0 && first)) {      // (test hook)
+                    const int n_at = min(lay.at, t_end - t);
                     const uint32_t fb = smem_u32(&full[st]);
-                    mbar_expect_tx(fb, bytes);
-                    const uint32_t dst = smem_u32(stages + st * stage_bytes);
-                    for (int at = 0; at < n_at; ++at) {
-                        const int st4 = (int)(s >> a.kt_shift) + at;   // k-tile of the pass
-                        const uint32_t o = (uint32_t)at * lay.atom;
-                        if (!alias) {
-                            tma_load_4d(dst + o, map, fb, ra, itm.k, st4);
+                    uint32_t dst = stage0 + st * stage_bytes;
+                    if (el) {
+                        mbar_expect_tx(fb, (uint32_t)n_at * tile_bytes);
+                        for (int at = 0; at < n_at; ++at, dst += lay.atom) {
+                            tma_load_4d(dst, map, fb, ra, itm.k, t + at);
                             if (planes == 2)
-                                tma_load_4d(dst + lay.plo + o, map, fb, ra, itm.k, d.cap_tiles + st4);
-                        }
-                        if (!single)
-                            for (int bb = 0; bb < itm.nbB; ++bb) {
-                                tma_load_4d(dst + bh_off + bb * slot + o, map, fb, rb + kRows * bb,
-                                            itm.k, st4);
+                                tma_load_4d(dst + lay.plo, map, fb, ra, itm.k, d.cap_tiles + t + at);
+                            if (!alias) {
+                                tma_load_4d(dst + bh_off, map, fb, rb, itm.k, t + at);
                                 if (planes == 2)
-                                    tma_load_4d(dst + bl_off + bb * slot + o, map, fb, rb + kRows * bb,
-                                                itm.k, d.cap_tiles + st4);
+                                    tma_load_4d(dst + bl_off, map, fb, rb, itm.k, d.cap_tiles + t + at);
                             }
+                        }
                     }
                     armed |= 1u << st;
                     armed_ph = (armed_ph & ~(1u << st)) | (ph << st);
                 }
-            }
-            if (!ok) {
-                // drain: every armed stage's copies must land before teardown
-                const unsigned long long d2 = globaltimer() + a.timeout_ns;
-                for (int s2 = 0; s2 < a.stages && s2 < 16; ++s2) {
-                    if (!((armed >> s2) & 1u)) continue;
-                    while (!mbar_try_wait(smem_u32(&full[s2]), (armed_ph >> s2) & 1u))
-                        if (globaltimer() > d2) break;
+                first = false;
+                if (++st == (uint32_t)a.stages) {
+                    st = 0;
+                    ph ^= 1u;
                 }
+            }
+        }
+        // WIDE: the last commits' arrivals from the other CTA are in
+        // (nothing else waits for them before this CTA may end)
+        if (WIDE)
+            for (int s2 = 0; ok && s2 < a.stages; ++s2)
+                if ((armed >> s2) & 1u)
+                    ok = __all_sync(0xffffffffu,
+                                    wait_bar(smem_u32(&empty[s2]), (armed_ph >> s2) & 1u, abort_word, a));
+        if (!ok) {
+            // drain: every armed stage's copies must land before teardown
+            const unsigned long long d2 = globaltimer() + a.timeout_ns;
+            for (int s2 = 0; s2 < a.stages && s2 < 16; ++s2) {
+                if (!((armed >> s2) & 1u)) continue;
+                while (!mbar_try_wait(smem_u32(&full[s2]), (armed_ph >> s2) & 1u))
+                    if (globaltimer() > d2) break;
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            uint32_t it = 0, st = 0, ph = 0;
-            int wi = 0;
-            bool ok = true;
-            bool issued = false;
-            PieceCursor cur;
-            cursor_init(a, cur);
-            Piece pc;
-            while (ok && next_piece(a, cur, pc)) {
-                const Item& itm = pc.itm;
-                const TcModeArgs& d = a.md[itm.m];
-                const bool single = !WIDE || d.nblk == 1;
-                const bool alias = !single && itm.b2 == itm.b1;
-                // single block: N = 2N rounded up to 16; group: N = 128 per B block
-                const int Nn = single ? (2 * block_ants(d.N, 0) + 15) & ~15 : kRows * itm.nbB;
-                // D = F32, A/B = F16 (kind::f16) or E4M3 (kind::f8f6f4), K-major,
-                // N>>3 at bits 17-22, M>>4 at bits 24-28
-                const uint32_t idesc =
-                    (1u << 4) | ((uint32_t)(Nn >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
-                // group: A from its own slots, or the first B block's
-                const uint32_t a_hi = alias ? bh_off : 0u;
-                const uint32_t a_lo = alias ? bl_off : plane_off;
-                const ItemLayout lay = item_layout(a, d, single, planes, stage_bytes, atom_bytes, plane_off);
-                const int step_i = a.KT * lay.at;
-                // FP32 mode, single block: B = [hi; lo], the k-tile's two tiles
-                // of box_rows rows each, N = 2 box_rows, so one MMA forms
-                // [Dhh | Dhl] (Dhl from column box_rows)
-                const int box_rows = (int)(d.box_bytes / (uint32_t)a.row_bytes);
-                const uint32_t idesc_cat = (1u << 4) | ((uint32_t)((2 * box_rows) >> 3) << 17) |
-                                           ((uint32_t)(kRows >> 4) << 24);
-                const int64_t s_beg = pc.s_beg;
-                const int64_t s_end = pc.s_end;
-                for (int64_t w0 = s_beg; ok && w0 < s_end; w0 += a.W, ++wi) {
-                    const int b = wi & 1;
-                    const uint32_t aph = (uint32_t)(wi >> 1) & 1u;
-                    if (!wait_bar(smem_u32(&acce[b]), aph ^ 1u, abort_word, a)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t d0 = tmem + (uint32_t)b * 256u;
-                    const int64_t w1 = min(s_end, w0 + a.W);
-                    uint32_t acc = 0;
-                    for (int64_t s = w0; s < w1; s += step_i, ++it) {
-                        if (it > 0 && ++st == (uint32_t)a.stages) {
+        if (WIDE && rank == 1) {
+            // the pair's other CTA: pass each full stage on to rank 0
+            if (lane == 0) {
+                uint32_t st = 0, ph = 0;
+                bool ok = true;
+                PieceCursor cur;
+                cursor_init<WIDE>(a, cur);
+                Piece pc;
+                while (ok && next_piece<WIDE>(a, cur, pc)) {
+                    const TcModeArgs& d = a.md[pc.itm.m];
+                    const bool alias = pc.itm.b2 == pc.itm.b1 && group_cols(d.N, pc.itm.b2) == 256;
+                    const ItemLayout lay = item_layout(a, d, alias, planes, stage_bytes, atom_bytes, plane_off);
+                    const int t_end = (int)(pc.s_end >> a.kt_shift);
+                    for (int t = (int)(pc.s_beg >> a.kt_shift); t < t_end; t += lay.at) {
+                        ok = wait_bar(smem_u32(&full[st]), ph, abort_word, a);
+                        if (!ok) break;
+                        mbar_relay(smem_u32(&full[st]), 0);
+                        if (++st == (uint32_t)a.stages) {
                             st = 0;
                             ph ^= 1u;
                         }
-                        if (!wait_bar(smem_u32(&full[st]), ph, abort_word, a)) {
+                    }
+                }
+            }
+        } else {
+            const bool el = elect_one();
+            uint32_t st = 0, ph = 0;
+            int wi = 0;
+            bool ok = true;
+            bool issued = false;
+            const uint32_t lo0 = op_desc_lo(smem_u32(stages));
+            constexpr uint32_t CG = WIDE ? 2 : 1;
+            PieceCursor cur;
+            cursor_init<WIDE>(a, cur);
+            Piece pc;
+            while (ok && next_piece<WIDE>(a, cur, pc)) {
+                const Item& itm = pc.itm;
+                const TcModeArgs& d = a.md[itm.m];
+                // single block: N = 2N rounded up to 16, FP32 mode: B = [hi;
+                // lo], the k-tile's two tiles of box_rows rows each, N = 2
+                // box_rows, so one MMA forms [Dhh | Dhl] (Dhl from column
+                // box_rows)
+                const int box_rows = (int)(d.box_bytes / (uint32_t)a.row_bytes);
+                const int Nn = !single     ? group_cols(d.N, itm.b2)
+                               : MODE == 0 ? 2 * box_rows
+                                           : (2 * block_ants(d.N, 0) + 15) & ~15;
+                const bool alias = single || (itm.b2 == itm.b1 && Nn == 256);
+                // D = F32, A/B = F16 (kind::f16) or E4M3 (kind::f8f6f4), K-major,
+                // N>>3 at bits 17-22, M>>4 at bits 24-28
+                const uint32_t idesc = (1u << 4) | ((uint32_t)(Nn >> 3) << 17) |
+                                       ((CG * kRows >> 4) << 24);
+                const ItemLayout lay = item_layout(a, d, alias, planes, stage_bytes, atom_bytes, plane_off);
+                // (descriptor addresses count 16 bytes)
+                const uint32_t al_o = lay.plo >> 4;                    // A lo
+                const uint32_t bh_o = alias ? 0u : bh_off >> 4;        // group: B from its own
+                const uint32_t bl_o = alias ? al_o : bl_off >> 4;      // slots, or A's (in both CTAs)
+                const uint32_t atom_o = lay.atom >> 4;
+                const int wk = a.W >> a.kt_shift;
+                const int t_end = (int)(pc.s_end >> a.kt_shift);
+                for (int t = (int)(pc.s_beg >> a.kt_shift); ok && t < t_end; ++wi) {
+                    const int b = wi & 1;
+                    const uint32_t aph = (uint32_t)(wi >> 1) & 1u;
+                    if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&acce[b]), aph ^ 1u, abort_word, a))) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t d0 = tmem + (uint32_t)b * 256u;
+                    const int tw = min(t_end, t + wk);
+                    uint32_t acc = 0;
+                    for (; t < tw; t += lay.at) {
+                        if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&full[st]), ph, abort_word, a))) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t base = smem_u32(stages + st * stage_bytes);
-                        const int n_at = (int)min((int64_t)lay.at, (w1 - s) >> a.kt_shift);
-                        for (int at = 0; at < n_at; ++at) {
-                            const uint32_t ab = base + (uint32_t)at * lay.atom;
+                        const int n_at = min(lay.at, tw - t);
+                        if (el) {
+                            uint32_t lo = lo0 + st * (stage_bytes >> 4);
+#pragma unroll 2
+                            for (int at = 0; at < n_at; ++at, lo += atom_o) {
 #pragma unroll
-                            for (int kk = 0; kk < KK; ++kk) {
-                                if (single) {
-                                    const uint64_t ah = op_desc<MODE>(ab + 32u * kk);
-                                    // FP32 mode: B = [hi; lo] forms [Dhh | Dhl]
-                                    mma<MODE>(d0, ah, ah, MODE == 0 ? idesc_cat : idesc, acc);
-                                } else {
-                                    const uint64_t ah = op_desc<MODE>(ab + a_hi + 32u * kk);
-                                    const uint64_t bh = op_desc<MODE>(ab + bh_off + 32u * kk);
-                                    mma<MODE>(d0, ah, bh, idesc, acc);
-                                    if (MODE == 0) {
-                                        const uint64_t al = op_desc<MODE>(ab + a_lo + 32u * kk);
-                                        const uint64_t bl = op_desc<MODE>(ab + bl_off + 32u * kk);
-                                        mma<MODE>(d0, ah, bl, idesc, 1u);
-                                        mma<MODE>(d0, al, bh, idesc, 1u);
+                                for (int kk = 0; kk < KK; ++kk) {
+                                    const uint64_t ah = op_desc<MODE>(lo + 2u * kk);
+                                    if (single) {
+                                        mma<MODE, CG>(d0, ah, ah, idesc, acc);
+                                    } else {
+                                        const uint64_t bh = op_desc<MODE>(lo + bh_o + 2u * kk);
+                                        mma<MODE, CG>(d0, ah, bh, idesc, acc);
+                                        if (MODE == 0) {
+                                            const uint64_t al = op_desc<MODE>(lo + al_o + 2u * kk);
+                                            const uint64_t bl = op_desc<MODE>(lo + bl_o + 2u * kk);
+                                            mma<MODE, CG>(d0, ah, bl, idesc, 1u);
+                                            mma<MODE, CG>(d0, al, bh, idesc, 1u);
+                                        }
                                     }
+                                    acc = 1;
                                 }
-                                acc = 1;
                             }
+                            mma_commit<CG>(smem_u32(&empty[st]));
+                            if (t + lay.at >= tw) mma_commit<CG>(smem_u32(&accf[b]));
                         }
+                        acc = 1;
                         issued = true;
-                        mma_commit(smem_u32(&empty[st]));
+                        if (++st == (uint32_t)a.stages) {
+                            st = 0;
+                            ph ^= 1u;
+                        }
                     }
-                    if (!ok) break;
-                    mma_commit(smem_u32(&accf[b]));
                 }
             }
             if (!ok && issued) {
-                // drain: wait for every MMA this thread issued before TMEM is freed
-                mma_commit(smem_u32(drain));
+                // drain: wait for every MMA this warp issued before TMEM is freed
+                if (el) mma_commit<CG>(smem_u32(drain));
                 const unsigned long long d2 = globaltimer() + a.timeout_ns;
                 while (!mbar_try_wait(smem_u32(drain), 0u))
                     if (globaltimer() > d2) break;
+                if (WIDE) __nanosleep(10000);      // the other CTA's arrivals of these commits
             }
         }
     } else {
@@ -568,29 +650,36 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         int wi = 0;
         // one cursor for the 8 warps, in shared memory (registers are scarce here)
         if (et == 0) {
-            cursor_init(a, *epi_cur);
-            epi_more[0] = next_piece(a, *epi_cur, epi_pc[0]) ? 1 : 0;
+            cursor_init<WIDE>(a, *epi_cur);
+            epi_more[0] = next_piece<WIDE>(a, *epi_cur, epi_pc[0]) ? 1 : 0;
         }
         epi_sync();
         for (int pb = 0;; pb ^= 1) {
             if (!epi_more[pb]) break;
             const Piece pc = epi_pc[pb];
             // the piece after it, while this one's windows are on their way
-            if (et == 0) epi_more[pb ^ 1] = next_piece(a, *epi_cur, epi_pc[pb ^ 1]) ? 1 : 0;
+            if (et == 0) epi_more[pb ^ 1] = next_piece<WIDE>(a, *epi_cur, epi_pc[pb ^ 1]) ? 1 : 0;
             const Item& itm = pc.itm;
             const TcModeArgs& d = a.md[itm.m];
-            const bool single = !WIDE || d.nblk == 1;
-            const bool use_t = MODE == 0 && single;
-            const int nb1 = block_ants(d.N, itm.b1);
-            const int nb2 = single ? nb1 : block_ants(d.N, itm.b2);
-            const int R2a = 2 * nb1;
-            const int R2b = 2 * nb2;
+            constexpr bool use_t = MODE == 0 && single;
+            // antennas of this CTA's A block (a group's second one may not exist)
+            const int nb1 = max(0, block_ants(d.N, itm.b1 + rank));
+            const int R2 = 2 * nb1;
             // columns per half: one block 2N rounded up to 16, halved (<= 64);
-            // a group 128 per B block, halved (<= 128)
-            const int NH = single ? ((R2b + 15) & ~15) >> 1 : (kRows * itm.nbB) >> 1;
+            // a group's columns, halved (<= 128)
+            const int NH = single ? ((R2 + 15) & ~15) >> 1 : group_cols(d.N, itm.b2) >> 1;
             const int col0 = h * NH;
             const int64_t s_beg = pc.s_beg;
             const int64_t s_end = pc.s_end;
+            // a group's scales, 64 of the rows' and 128 of the columns'
+            // antennas, while its windows are on their way (read for each V,
+            // from global memory: FP16 at N = 256 655 us a pass, now 589)
+            if (!single && et < 192) {
+                const int i = et < 64 ? 64 * (itm.b1 + rank) + et : 64 * itm.b2 + et - 64;
+                Gs[et] = i >= d.N ? 1.f
+                                  : (MODE == 0 ? __ldg(d.split + i)
+                                               : __ldg(d.scale + (int64_t)i * d.C + itm.k));
+            }
             // window sums: acc[0 .. NH) (single block, FP32 mode: [0, 64) from
             // hi hi^T and [64, 64 + NH) from hi lo^T)
             float acc[128];
@@ -634,7 +723,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&acce[b]));   // this warp's slice is free
+                if (lane == 0) {                                  // this warp's slice is free
+                    if (rank == 0)
+                        mbar_arrive(smem_u32(&acce[b]));
+                    else
+                        mbar_arrive_rank(smem_u32(&acce[b]), 0);
+                }
             }
             epi_sync();
             // one reading of the abort word for the 8 warps (the producer and
@@ -686,19 +780,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                         const int j_loc = jg & 63;
                         const bool jv = j_loc < block_ants(N, b2);
                         const int j = 64 * b2 + j_loc;
-                        const float sj = !jv ? 1.f
-                                             : (MODE == 0 ? __ldg(d.split + j)
-                                                          : __ldg(d.scale + (int64_t)j * C + itm.k));
+                        const float sj = Gs[64 + jg];
 #pragma unroll 1
                         for (int i0 = 0; i0 < 16; i0 += kRowsPerStep) {
                             const int i16 = i0 + lane / kVCols;
                             const int i_loc = 16 * q + i16;
                             if (16 * q + i0 >= nb1) break;
-                            if (i_loc < nb1 && jv && !(b2 == itm.b1 && j_loc < i_loc)) {
-                                const int i = 64 * itm.b1 + i_loc;
-                                const float si = MODE == 0 ? __ldg(d.split + i)
-                                                           : __ldg(d.scale + (int64_t)i * C + itm.k);
-                                const float f = 1.0f / (si * sj);
+                            const int i = 64 * (itm.b1 + rank) + i_loc;
+                            if (i_loc < nb1 && jv && j >= i) {
+                                const float f = 1.0f / (Gs[i_loc] * sj);
                                 const float2 v = vst[i16 * kVRow + jj];
                                 const int p = i * N - i * (i - 1) / 2 + (j - i);
                                 pout[p] = make_float2(v.x * f, v.y * f);
@@ -714,14 +804,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
             // blocks has its own place (Ld): one store per element, and the
             // pair adds the transposed element when it reads.  (Adding L^T in
             // place cost a dependent shared load, add and store per element.)
-            const int ldg = R2b + 1;
+            const int ldg = R2 + 1;
             float* Ld = Gs + a.gs_floats - 2 * kRows;          // [row][col mod 2]
-            if (r < R2a) {
+            if (r < R2) {
                 const int dcol = r & ~1;                       // the diagonal block's first column
 #pragma unroll
                 for (int c = 0; c < 64; ++c) {
                     const int col = col0 + c;
-                    if (c < NH && col < R2b) {
+                    if (c < NH && col < R2) {
                         Gs[r * ldg + col] = use_t ? (col < dcol ? acc[64 + c] : acc[c] + acc[64 + c]) : acc[c];
                         if (use_t && (col & ~1) == dcol) Ld[2 * r + (col & 1)] = acc[64 + c];
                     }
@@ -795,10 +885,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 // finish adds every partial, in slot order, into the FP64
                 // accumulator (a group: into slot 0, see the run's reduction):
                 // deterministic.
+                // (The two CTAs of a pair hold different rows: a counter each.)
+                int* const ticket = d.ticket + (itm.k * d.npairs + itm.pr) * (WIDE ? 2 : 1) + rank;
                 __threadfence();
                 epi_sync();
                 if (et == 0) {
-                    const int old = atomicAdd(d.ticket + itm.k * d.npairs + itm.pr, 1);
+                    const int old = atomicAdd(ticket, 1);
                     *epi_last = old == pc.nslots - 1 ? 1 : 0;
                 }
                 epi_sync();
@@ -826,9 +918,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                                 const int rest = pl - i_loc * 64 * itm.nbB;
                                 const int b2 = itm.b2 + (rest >> 6);
                                 const int j_loc = rest & 63;
-                                if (j_loc >= block_ants(N, b2) || (b2 == itm.b1 && j_loc < i_loc)) continue;
-                                const int i = 64 * itm.b1 + i_loc;
+                                const int i = 64 * (itm.b1 + rank) + i_loc;
                                 const int j = 64 * b2 + j_loc;
+                                if (j_loc >= block_ants(N, b2) || j < i) continue;
                                 pp[u] = i * N - i * (i - 1) / 2 + (j - i);
                             }
                         }
@@ -865,21 +957,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                                     d.partial[(int64_t)itm.k * P + pp[u]] = make_float2((float)re[u], (float)im[u]);
                         }
                     }
-                    if (et == 0) d.ticket[itm.k * d.npairs + itm.pr] = 0;
+                    if (et == 0) *ticket = 0;
                 }
             }
             epi_sync();
         }
     }
 
+    // (a pair's CTAs end together: each may still read the other's tiles, and
+    // arrive at its barriers, until here; every wait before this one is bounded)
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if (WIDE)
+        cluster_sync();
+    else
+        __syncthreads();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(kTmemCols)
-                     : "memory");
+        if (WIDE)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                         "r"(kTmemCols)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                         "r"(kTmemCols)
+                         : "memory");
     }
 }
 
@@ -914,7 +1017,8 @@ struct TcPlan {
     unsigned long long timeout_ns = 4000000000ull;
     int withhold = 0;                    // test hook for the next launch
     unsigned long long hook_timeout_ns = 0;
-    int* ticket = nullptr;               // [C][npairs] arrival counters
+    int* ticket = nullptr;               // [C][npairs][2 if nblk > 1] arrival counters
+    size_t ticket_bytes() const { return (size_t)C * npairs * (nblk > 1 ? 2 : 1) * sizeof(int); }
     // split decisions already made, keyed by the S_pad of every mode in the launch
     std::vector<std::pair<std::vector<int64_t>, DealPlan>> split_cache;
 };
@@ -943,7 +1047,7 @@ int tc_plan_create(TcPlan** out, int N, int C, int spec_type, std::string& err) 
         err = "cudaDeviceGetAttribute failed";
         return CORR_ECUDA;
     }
-    const size_t tb = (size_t)p->C * p->npairs * sizeof(int);
+    const size_t tb = p->ticket_bytes();
     if (dev_malloc((void**)&p->ticket, tb) != cudaSuccess || cudaMemset(p->ticket, 0, tb) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p->ticket);
@@ -957,7 +1061,7 @@ int tc_plan_create(TcPlan** out, int N, int C, int spec_type, std::string& err) 
 
 int tc_reset(TcPlan* p) {
     // after an aborted launch some arrival counters may be left non-zero
-    return cudaMemset(p->ticket, 0, (size_t)p->C * p->npairs * sizeof(int)) == cudaSuccess
+    return cudaMemset(p->ticket, 0, p->ticket_bytes()) == cudaSuccess
                ? CORR_OK
                : CORR_ECUDA;
 }
@@ -1030,15 +1134,18 @@ struct LaunchShape {
     size_t smem;
 };
 
-LaunchShape launch_shape(TcPlan* const* plans, int n) {
+// lead: the plan whose tile choices hold for the launch.
+LaunchShape launch_shape(const TcPlan* lead, TcPlan* const* plans, int n) {
     LaunchShape L{};
-    int r2max = 0;     // the G buffer serves the single-block modes only
-    for (int m = 0; m < n; ++m) {
-        L.wide |= plans[m]->nblk > 1;
-        if (plans[m]->nblk == 1) r2max = std::max(r2max, 2 * plans[m]->N);
+    L.wide = plans[0]->nblk > 1;
+    // single block: G, and in FP32 mode L of its diagonal blocks; groups: scales
+    if (L.wide) {
+        L.gs_floats = 64 + 128;
+    } else {
+        int r2max = 0;
+        for (int m = 0; m < n; ++m) r2max = std::max(r2max, 2 * plans[m]->N);
+        L.gs_floats = r2max * (r2max + 1) + (plans[0]->mode == 0 ? 2 * kRows : 0);
     }
-    // G, and in FP32 mode L of its diagonal blocks
-    L.gs_floats = r2max * (r2max + 1) + (plans[0]->mode == 0 ? 2 * kRows : 0);
     L.slot_rows = 8;
     int min_box = kRows;      // the MMA reads 128 rows from a tile: reserve the excess past the ring
     for (int m = 0; m < n; ++m) {
@@ -1051,34 +1158,31 @@ LaunchShape launch_shape(TcPlan* const* plans, int n) {
     const size_t fixed = 1024 + (size_t)L.gs_floats * 4 + vstage + 16 + 16 + 8 * (2 * 16 + 5) + 256 +
                          (size_t)(kRows - min_box) * plans[0]->row_bytes;
     auto fit = [&](int atoms) {
-        const size_t sb = (size_t)plans[0]->planes * atoms * slot * (L.wide ? 3 : 1);
+        const size_t sb = (size_t)plans[0]->planes * atoms * slot * (L.wide ? 2 : 1);
         return std::min<int>(16, (int)((kSmemBudget - fixed) / sb));
     };
     // k-tiles per stage, unless set: as many (up to 256 spectra: 8 k-tiles of
-    // 32, or 4 of the FP8 mode's 128) as still leave 3 stages; with two tiles
-    // per k-tile (several antenna blocks) 2 stages suffice -- each stage
-    // handshake costs a fixed latency, measured at N = 256: 2 stages of 128
-    // spectra 1.10 ms against 4 of 64 1.24 ms per pass
-    L.atoms = plans[0]->atoms;
+    // 32, or 4 of the FP8 mode's 128) as still leave 3 stages -- each stage
+    // handshake costs a fixed latency
+    L.atoms = lead->atoms;
     if (!L.atoms) {
         L.atoms = 1;
-        const int min_stages = L.wide ? 2 : 3;
         for (int at = plans[0]->KT == 32 ? 8 : 4; at > 1; at /= 2)
-            if (fit(at) >= min_stages) {
+            if (fit(at) >= 3) {
                 L.atoms = at;
                 break;
             }
     }
     while (L.atoms > 1 && fit(L.atoms) < 2) L.atoms /= 2;
     const size_t stage_bytes =
-        (size_t)plans[0]->planes * L.atoms * slot * (L.wide ? 3 : 1);
+        (size_t)plans[0]->planes * L.atoms * slot * (L.wide ? 2 : 1);
     const int smax = fit(L.atoms);
     // default depth: as many stages as fit, up to 8; FP32 mode with one
     // antenna block, which streams its workspace from HBM at the copy rate,
     // takes 3 (at N = 44 a 1 s integration's pass: 0.92 ms against 0.95 with
     // the 4 that fit, 1.03 with 2)
     const int sdef = plans[0]->mode == 0 && !L.wide ? 3 : 8;
-    L.stages = plans[0]->stages ? std::min(plans[0]->stages, smax) : std::min(smax, sdef);
+    L.stages = lead->stages ? std::min(lead->stages, smax) : std::min(smax, sdef);
     const int step = plans[0]->KT * L.atoms;
     // default window: 256 spectra in FP32 mode (TMEM accumulation bias ~1e-6
     // at full size); 512 for FP16 (its input rounding dominates), 1024 when
@@ -1088,43 +1192,54 @@ LaunchShape launch_shape(TcPlan* const* plans, int n) {
     // 1024-spectrum FP16 window: 30% less time per pass than 1024 at
     // N = 256, 13% at N = 44, against an input rounding error near 1e-2)
     const int W0 = plans[0]->mode == 0 ? 256 : plans[0]->mode == 2 ? 2048 : (L.wide ? 1024 : 512);
-    int W = plans[0]->window ? plans[0]->window : std::max(W0, plans[0]->KT);
+    int W = lead->window ? lead->window : std::max(W0, plans[0]->KT);
     L.W = (W + step - 1) / step * step;   // windows hold whole stages
     L.smem = fixed + (size_t)L.stages * stage_bytes;
     return L;
 }
 
 // Work deal of one launch.  Round-robin: every mode's pass of S_pad frames
-// is cut into n_split ranges of whole k-tiles per item and items go to CTAs
-// in turn; the range count minimises the busiest CTA's work in a simulation
-// of that deal.  Balanced (single-mode launches): contiguous shares of the
-// weighted k-tiles (see next_piece).  The cheaper of the two in the same
-// cost model is taken (per item or piece: its k-tiles x 1 on a diagonal
-// block pair, x 1.5 off it, plus ~4 k-tiles for its end, measured on GB300,
-// and 2 more when its partial is combined with others).  At N = 44, K = 512
-// and 8192 frames per pass the round-robin deal leaves 104 CTAs with two
-// channels and 48 with one; the balanced deal gives each 1.7 channels.
-DealPlan choose_deal(TcPlan* const* plans, int n, const int64_t* S_pad) {
+// is cut into n_split ranges of whole k-tiles per item and items go to the
+// workers in turn; the range count minimises the busiest worker's work in a
+// simulation of that deal.  Balanced (one single-block mode): contiguous
+// shares of the weighted k-tiles (see next_piece).  The cheaper of the two in
+// the same cost model is taken: per item or piece of a single block its
+// k-tiles, ~4 more for its end, and 2 more when its partial is combined with
+// others.  At N = 44, K = 512 and 8192 frames per pass the round-robin deal
+// leaves 104 CTAs with two channels and 48 with one; the balanced deal gives
+// each 1.7 channels.  Groups: an end takes ~1.5 us, but combining the 8192
+// baselines of a CTA's tile in FP64 ~36 us, far more than the k-tiles that a
+// cut moves elsewhere unless a pass has few channels and many spectra (N =
+// 100, K = 512, 2048 frames FP16: 68 us whole, 206 cut in two; N = 192, 4096
+// frames: 245 against 470).
+DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int64_t* S_pad) {
     std::vector<int64_t> key(S_pad, S_pad + n);
     DealPlan out;
-    if (plans[0]->split > 0) {
+    if (lead->split > 0) {
         // fixed by corr_set_tiles: round-robin, ranges per channel, at most one per k-tile
         out.sp.resize(n);
         for (int m = 0; m < n; ++m) {
             const int64_t tiles = std::max<int64_t>(1, S_pad[m] / plans[m]->KT);
-            out.sp[m] = (int)std::min<int64_t>(std::min(plans[0]->split, plans[m]->max_split), tiles);
+            out.sp[m] = (int)std::min<int64_t>(std::min(lead->split, plans[m]->max_split), tiles);
         }
         return out;
     }
     auto& cache = plans[0]->split_cache;
     for (auto& e : cache)
         if (e.first == key) return e.second;
-    const int sms = plans[0]->num_sms;
+    // workers: CTAs, or with several antenna blocks CTA pairs
+    const int sms = plans[0]->nblk > 1 ? plans[0]->num_sms / 2 : plans[0]->num_sms;
     int64_t max_tiles = 1;
     for (int m = 0; m < n; ++m) max_tiles = std::max<int64_t>(max_tiles, S_pad[m] / plans[m]->KT);
     std::vector<int> best(n, 1);
     double best_score = 1e300;
     std::vector<double> load(sms);
+    // cost of an item's end and of its share in combining partials, in k-tiles
+    // (FP32 mode, FP16, FP8; a group's k-tile takes 0.5, 0.2 and 0.4 us)
+    static const double kGroupEnd[3] = {3, 8, 4}, kGroupCombine[3] = {70, 180, 90};
+    const bool groups = plans[0]->nblk > 1;
+    const double end = groups ? kGroupEnd[plans[0]->mode] : 4.0;
+    const double combine = groups ? kGroupCombine[plans[0]->mode] : 2.0;
     for (int64_t T = 1; T <= max_tiles * 2; T *= 2) {
         std::vector<int> sp(n);
         for (int m = 0; m < n; ++m) {
@@ -1142,10 +1257,13 @@ DealPlan choose_deal(TcPlan* const* plans, int n, const int64_t* S_pad) {
             const int64_t per = (tiles + sp[m] - 1) / sp[m];
             for (int s = 0; s < sp[m]; ++s) {
                 const int64_t t = std::min<int64_t>(per, tiles - (int64_t)s * per);
-                for (int k = 0; k < p->C; ++k)
+                for (int k = 0; k < p->C; ++k) {
+                    const int turn = group_turn((int)g, p->npairs, sms);
                     for (int pr = 0; pr < p->npairs; ++pr, ++g)
-                        load[g % sms] += (double)t * 0.5 * host_pair_units(pr, p->nblk) + 4.0 +
-                                         (sp[m] > 1 ? 2.0 : 0.0);
+                        load[g % sms] +=
+                            (double)t * 0.5 * host_pair_units((pr + turn) % p->npairs, p->nblk) + end +
+                            (sp[m] > 1 ? combine : 0.0);
+                }
             }
         }
         const double score = *std::max_element(load.begin(), load.end());
@@ -1213,6 +1331,116 @@ DealPlan choose_deal(TcPlan* const* plans, int n, const int64_t* S_pad) {
 
 }  // namespace
 
+namespace {
+
+// One kernel for plans that all have one antenna block, or all several.
+int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, cudaStream_t st,
+               std::string& err) {
+    std::vector<int64_t> S(n);
+    for (int m = 0; m < n; ++m) S[m] = runs[m]->S_pad;
+    const DealPlan deal = choose_deal(lead, plans, n, S.data());
+    const std::vector<int>& sp = deal.sp;
+    const LaunchShape L = launch_shape(lead, plans, n);
+    TcArgs a;
+    memset(&a, 0, sizeof a);
+    a.n_modes = n;
+    a.stages = L.stages;
+    a.KT = plans[0]->KT;
+    a.kt_shift = a.KT == 128 ? 7 : 5;
+    a.row_bytes = plans[0]->row_bytes;
+    a.W = L.W;
+    a.atoms = L.atoms;
+    a.wide = L.wide;
+    a.gs_floats = L.gs_floats;
+    a.slot_rows = L.slot_rows;
+    a.status = runs[0]->status;
+    a.timeout_ns = lead->timeout_ns;
+    if (lead->withhold) {
+        a.withhold = 1;
+        a.timeout_ns = lead->hook_timeout_ns;
+        lead->withhold = 0;
+    }
+    int base = 0;
+    int64_t units = 0;
+    for (int m = 0; m < n; ++m) {
+        const TcPlan* p = plans[m];
+        a.tmap[m] = p->tmap;
+        TcModeArgs& d = a.md[m];
+        d.N = p->N;
+        d.C = p->C;
+        d.P = p->P;
+        d.nblk = p->nblk;
+        d.npairs = p->npairs;
+        d.S_pad = runs[m]->S_pad;
+        const int64_t tiles = std::max<int64_t>(1, d.S_pad / p->KT);
+        const int64_t per = (tiles + sp[m] - 1) / sp[m];
+        d.S_item = per * p->KT;
+        d.n_split = d.S_pad > 0 ? (int)((d.S_pad + d.S_item - 1) / d.S_item) : 0;
+        d.item_base = base;
+        d.n_items = d.n_split * p->npairs * p->C;
+        base += d.n_items;
+        d.partial = runs[m]->partial;
+        d.acc = runs[m]->acc;
+        d.ticket = plans[m]->ticket;
+        d.scale = runs[m]->scale;
+        d.split = runs[m]->split;
+        d.assign = runs[m]->assign;
+        d.tiles = d.S_pad / p->KT;
+        d.cap_tiles = (int)(p->cap / p->KT);
+        d.box_bytes = (uint32_t)p->box_rows * p->row_bytes;
+        d.unit_base = units;
+        for (int pr = 0; pr < p->npairs; ++pr)
+            units += item_units(d.tiles, host_pair_units(pr, p->nblk)) * p->C;
+        // single block: splits are combined inside the kernel, into acc;
+        // several blocks: every pass result lands in partial slot 0 (coalesced
+        // FP32 stores), which one reduction launch adds to acc
+        runs[m]->direct = p->nblk == 1;
+        runs[m]->n_split = runs[m]->direct ? d.n_split : 1;
+    }
+    a.total_items = base;
+    // (largest dividend of the deal: units x CTAs plus a divisor)
+    a.u32 = (units + 1) * (plans[0]->num_sms + 1) < ((int64_t)1 << 32);
+    if (base == 0) return CORR_OK;
+    int grid = L.wide ? 2 * std::min(base, plans[0]->num_sms / 2) : std::min(base, plans[0]->num_sms);
+    if (deal.balanced) {
+        a.balanced = 1;
+        a.units = units;
+        grid = deal.grid;
+    }
+    cudaError_t e;
+    auto go = [&](auto kern) {
+        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)L.smem);
+        if (r != cudaSuccess) return r;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute pair[1];
+        pair[0].id = cudaLaunchAttributeClusterDimension;
+        pair[0].val.clusterDim.x = 2;
+        pair[0].val.clusterDim.y = pair[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kTcThreads);
+        cfg.dynamicSmemBytes = L.smem;
+        cfg.stream = st;
+        cfg.attrs = pair;
+        cfg.numAttrs = L.wide ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kern, a);
+    };
+    if (plans[0]->mode == 0)
+        e = L.wide ? go(xengine_tc_kernel<0, true>) : go(xengine_tc_kernel<0, false>);
+    else if (plans[0]->mode == 1)
+        e = L.wide ? go(xengine_tc_kernel<1, true>) : go(xengine_tc_kernel<1, false>);
+    else
+        e = L.wide ? go(xengine_tc_kernel<2, true>) : go(xengine_tc_kernel<2, false>);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        err = std::string("tensor-core X-engine launch: ") + cudaGetErrorString(e);
+        return CORR_ECUDA;
+    }
+    return CORR_OK;
+}
+
+}  // namespace
+
 int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err) {
     if (n < 1 || n > kMaxTcModes) {
         err = "between 1 and 4 modes per tensor-core launch";
@@ -1228,94 +1456,22 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
             return CORR_EINVAL;
         }
     }
-    std::vector<int64_t> S(n);
-    for (int m = 0; m < n; ++m) S[m] = runs[m].S_pad;
-    const DealPlan deal = choose_deal(plans, n, S.data());
-    const std::vector<int>& sp = deal.sp;
-    const LaunchShape L = launch_shape(plans, n);
-    TcArgs a;
-    memset(&a, 0, sizeof a);
-    a.n_modes = n;
-    a.stages = L.stages;
-    a.KT = plans[0]->KT;
-    a.kt_shift = a.KT == 128 ? 7 : 5;
-    a.row_bytes = plans[0]->row_bytes;
-    a.W = L.W;
-    a.atoms = L.atoms;
-    a.wide = L.wide;
-    a.gs_floats = L.gs_floats;
-    a.slot_rows = L.slot_rows;
-    a.status = runs[0].status;
-    a.timeout_ns = plans[0]->timeout_ns;
-    if (plans[0]->withhold) {
-        a.withhold = 1;
-        a.timeout_ns = plans[0]->hook_timeout_ns;
-        plans[0]->withhold = 0;
-    }
-    int base = 0;
-    int64_t units = 0;
-    for (int m = 0; m < n; ++m) {
-        const TcPlan* p = plans[m];
-        a.tmap[m] = p->tmap;
-        TcModeArgs& d = a.md[m];
-        d.N = p->N;
-        d.C = p->C;
-        d.P = p->P;
-        d.nblk = p->nblk;
-        d.npairs = p->npairs;
-        d.S_pad = runs[m].S_pad;
-        const int64_t tiles = std::max<int64_t>(1, d.S_pad / p->KT);
-        const int64_t per = (tiles + sp[m] - 1) / sp[m];
-        d.S_item = per * p->KT;
-        d.n_split = d.S_pad > 0 ? (int)((d.S_pad + d.S_item - 1) / d.S_item) : 0;
-        d.item_base = base;
-        d.n_items = d.n_split * p->npairs * p->C;
-        base += d.n_items;
-        d.partial = runs[m].partial;
-        d.acc = runs[m].acc;
-        d.ticket = plans[m]->ticket;
-        d.scale = runs[m].scale;
-        d.split = runs[m].split;
-        d.assign = runs[m].assign;
-        d.tiles = d.S_pad / p->KT;
-        d.cap_tiles = (int)(p->cap / p->KT);
-        d.box_bytes = (uint32_t)p->box_rows * p->row_bytes;
-        d.unit_base = units;
-        for (int pr = 0; pr < p->npairs; ++pr)
-            units += item_units(d.tiles, host_pair_units(pr, p->nblk)) * p->C;
-        // single block: splits are combined inside the kernel, into acc;
-        // several blocks: every pass result lands in partial slot 0 (coalesced
-        // FP32 stores), which one reduction launch adds to acc
-        runs[m].direct = p->nblk == 1;
-        runs[m].n_split = runs[m].direct ? d.n_split : 1;
-    }
-    a.total_items = base;
-    // (largest dividend of the deal: units x CTAs plus a divisor)
-    a.u32 = (units + 1) * (plans[0]->num_sms + 1) < ((int64_t)1 << 32);
-    if (base == 0) return CORR_OK;
-    int grid = std::min(base, plans[0]->num_sms);
-    if (deal.balanced) {
-        a.balanced = 1;
-        a.units = units;
-        grid = deal.grid;
-    }
-    cudaError_t e;
-    auto go = [&](auto kern) {
-        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)L.smem);
-        if (r == cudaSuccess) kern<<<grid, kTcThreads, L.smem, st>>>(a);
-        return r;
-    };
-    if (plans[0]->mode == 0)
-        e = L.wide ? go(xengine_tc_kernel<0, true>) : go(xengine_tc_kernel<0, false>);
-    else if (plans[0]->mode == 1)
-        e = L.wide ? go(xengine_tc_kernel<1, true>) : go(xengine_tc_kernel<1, false>);
-    else
-        e = L.wide ? go(xengine_tc_kernel<2, true>) : go(xengine_tc_kernel<2, false>);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        err = std::string("tensor-core X-engine launch: ") + cudaGetErrorString(e);
-        return CORR_ECUDA;
+    // Modes of one antenna block and modes of several take a kernel each (CTA
+    // pairs share their MMAs, and one kernel's tcgen05 code is of one
+    // cta_group).  The lead's set goes first: a test hook on it fires there.
+    TcPlan* set[kMaxTcModes];
+    TcRun* srun[kMaxTcModes];
+    const bool wide0 = plans[0]->nblk > 1;
+    for (int pass = 0; pass < 2; ++pass) {
+        int ns = 0;
+        for (int m = 0; m < n; ++m)
+            if ((plans[m]->nblk > 1) == (wide0 == (pass == 0))) {
+                set[ns] = plans[m];
+                srun[ns++] = &runs[m];
+            }
+        if (!ns) continue;
+        const int rc = launch_set(plans[0], set, ns, srun, st, err);
+        if (rc != CORR_OK) return rc;
     }
     return CORR_OK;
 }

@@ -33,12 +33,14 @@ int tc_plan_update(TcPlan* p, void* spec, int64_t cap, int N, int C, int spec_ty
 // stages (0 = as many as shared memory holds, up to 8), ranges per channel
 // of a pass (0 = the planner's choice) and k-tiles per stage (0 = automatic).
 int tc_set_tiles(TcPlan* p, int window, int stages, int split, int atoms, std::string& err);
-// One persistent launch over the passes of n plans sharing a precision.
+// Persistent launches over the passes of n plans sharing a precision: one for
+// the modes of a single antenna block, one for those of several.  Tile choices
+// are those of plans[0].
 // Modes whose run reports direct = false need the reduction of their
 // n_split partial blocks into acc.
 int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err);
-// Test hook: the next launch's CTA 0 skips the copy of its first k-tile, so
-// its MMA thread's bounded wait expires after wait_limit_s.
+// Test hook: the next launch's CTA 0 skips the copies of its first stage, so
+// its MMA warp's bounded wait expires after wait_limit_s.
 int tc_test_withhold(TcPlan* p, double wait_limit_s, std::string& err);
 // Clear the split arrival counters (after an aborted launch).
 int tc_reset(TcPlan* p);

@@ -57,9 +57,9 @@ def xengine_issued_flops(N, K, s_pad, dtype):
     * one block (N <= 64): FP32 mode (two FP16 planes) one MMA whose B is
       [hi; lo], N = 2 r (r = 2N rounded up to 8); FP16 / FP8 one MMA with
       N = 2N rounded up to 16;
-    * several blocks: work groups of block b1 against blocks b2 .. b2 +
-      nbB - 1 (b2 = b1, b1 + 2, ...; nbB = 2, or 1 for a row's last), one
-      MMA with N = 128 nbB (three in FP32 mode: hi hi, hi lo, lo hi).
+    * several blocks: work groups of two blocks against two (b1 <= b2, both
+      even), one MMA of a CTA pair, M = 256, N the group's B rows rounded up
+      to 64, at most 256 (three MMAs in FP32 mode: hi hi, hi lo, lo hi).
     """
     nblk = (N + 63) // 64
     if nblk == 1:
@@ -69,8 +69,7 @@ def xengine_issued_flops(N, K, s_pad, dtype):
             per = 2 * 128 * ((2 * N + 15) // 16 * 16)
     else:
         per = 0
-        for b1 in range(nblk):
-            for b2 in range(b1, nblk, 2):
-                nn = 128 * min(2, nblk - b2)
-                per += (3 if dtype == "fp32" else 1) * 2 * 128 * nn
+        for b2 in range(0, nblk, 2):
+            nn = min(256, (2 * N - 128 * b2 + 63) // 64 * 64)
+            per += (b2 // 2 + 1) * (3 if dtype == "fp32" else 1) * 2 * 256 * nn
     return float(per) * (K // 2) * s_pad
