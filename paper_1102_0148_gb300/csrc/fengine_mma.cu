@@ -15,13 +15,17 @@
 // product and every sum of a stage-1 accumulator is an exact multiple of
 // 2^-11 below 2^21 of them: the tensor core rounds nothing, and
 // y = fma(lo, 2^-12, hi) has one rounding.  (The elements are exact to 2^-24.)
+// For M >= 16 (K >= 512) stage 1 is folded first: even k1 take x[n1] + x[n1 +
+// N1/2], odd k1 the differences (exact, one packed add per pair of MMA
+// operands), which halves the matrix and its MMAs; an m-tile then holds k1 of
+// one parity.
 // Stage 2 is the twiddle and an M-point DFT per k1 on the FP32 pipes.  As y
 // comes from the real samples, k1 = 1 .. N1/2 - 1 gives X[k] for k < K/2 (k2 <
 // M/2) and conj X[K - k] for the rest: all channels but the multiples of N1/2
 // appear without a real-to-complex split.
 //
 // Fragment layouts make the exchange between the stages free.  Rows of an
-// m-tile are Re (row g) and Im (row g + 8) of k1 = 8 mt + g; the 8 columns are
+// m-tile are Re (row g) and Im (row g + 8) of 8 k1 (k1_of); the 8 columns are
 // 8 frames; one MMA set per n2.  A lane (g = lane / 4, c = lane % 4) thus ends
 // with y[k1][n2] of frames 2c and 2c + 1 for every n2, in registers: no shared
 // memory, no shuffles.  The sample operand wants, per lane, pairs of n1 of one
@@ -41,17 +45,19 @@
 // What bounds it: issue slots and register ports -- mma.sync and FP32
 // instructions do not overlap fully here (4 HMMA + 32 FFMA per warp take 1.4
 // times the longer of the two), so the stage-1 MMAs cost about a quarter of
-// the time -- at 12-16 warps per SM (64 accumulators per lane).  190-250 warp
-// instructions per 512 samples against 453 of the FP32 radix-16 kernel.
+// the time before the fold -- at 12-16 warps per SM (64 accumulators per
+// lane).  190-250 warp instructions per 512 samples (unfolded) against 453 of
+// the FP32 radix-16 kernel.
 // Measured per pass (GB300, before -> now):
 //   K = 256,  N = 64,  16384 frames: FP32 mode 4152 -> 230 us, FP16 4099 -> 179
 //             (before: the general radix-2 kernel, one frame at a time);
-//   K = 512,  N = 44,  16384 frames: FP16 337 -> 280 us, FP8 344 -> 285; FP32
-//             mode 350 -> 347 (bound by its 4 bytes per sample of output): the
-//             FP32 kernel stays there;
-//   K = 1024, N = 256, 4096 frames: FP16 1236 -> 1078 us; FP32 mode 1371 ->
-//             1362, the FP32 kernel stays;
-//   K = 2048, N = 64,  4096 frames: FP32 mode 1124 -> 987 us, FP16 1001 -> 727.
+//   K = 512,  N = 44,  16384 frames: FP16 337 -> 263 us (unfolded 284), FP8
+//             344 -> 274 (295); FP32 mode 346 against 369 here: the FP32
+//             kernel stays there;
+//   K = 1024, N = 256, 4096 frames: FP16 1236 -> 960 us (1130), FP8 977 (1062);
+//             FP32 mode 1374 against 1449 here, the FP32 kernel stays;
+//   K = 2048, N = 64,  4096 frames: FP16 1001 -> 695 us (728), FP8 700 (757),
+//             FP32 mode 1124 -> 901 (877).
 #include "corr_internal.h"
 #include "fengine_k512.cuh"
 #include "tc_ptx.cuh"
@@ -104,18 +110,28 @@ constexpr double cos_k(int m, int K) {
     return neg ? -v : v;
 }
 
-// A fragments (row-major m16 x k16) of the N1 x N1 stage-1 matrix, per m-tile,
-// k-tile, part (hi, lo 2^12) and lane.  PAIR: K = N1 (M = 1), where the two
+// Folded stage 1 (M >= 16): the matrix takes x[n1] + x[n1 + N1/2] for even k1
+// and x[n1] - x[n1 + N1/2] for odd k1, half the columns; m-tiles hold k1 of one
+// parity.
+constexpr bool folded(int M) { return M >= 16; }
+// k1 of row g of m-tile mt.
+__host__ __device__ constexpr int k1_of(bool fold, int mt, int g) {
+    return fold ? 16 * (mt >> 1) + 2 * g + (mt & 1) : 8 * mt + g;
+}
+
+// A fragments (row-major m16 x k16) of the stage-1 matrix, per m-tile, k-tile,
+// part (hi, lo 2^12) and lane.  PAIR: K = N1 (M = 1), where the two
 // samples of a pair come from the two nibbles of one byte and the odd one is
 // 16 times larger: its columns are divided by 16.
-template <int N1, bool PAIR>
+template <int N1, bool PAIR, bool FOLD>
 struct WFrag {
-    uint4 v[N1 / 16][N1 / 16][2][32];
+    static constexpr int KT = N1 / 16 / (FOLD ? 2 : 1);
+    uint4 v[N1 / 16][KT][2][32];
 };
 
-constexpr int w_part(int N1, int row16, int mt, int n1, int hl) {
+constexpr int w_part(int N1, bool fold, int row16, int mt, int n1, int hl) {
     const int g = row16 & 7, im = row16 >> 3;
-    const int k1 = 8 * mt + g;
+    const int k1 = k1_of(fold, mt, g);
     double w = 0.0;
     if (k1 == 0)
         w = im ? ((n1 & 1) ? -1.0 : 1.0) : 1.0;     // k1 = 0 and k1 = N1/2, both real
@@ -125,19 +141,19 @@ constexpr int w_part(int N1, int row16, int mt, int n1, int hl) {
     return hl ? round_abs((w * 2048.0 - hi) * 4096.0) : hi;
 }
 
-template <int N1, bool PAIR>
-constexpr WFrag<N1, PAIR> make_wfrag() {
-    WFrag<N1, PAIR> f{};
+template <int N1, bool PAIR, bool FOLD>
+constexpr WFrag<N1, PAIR, FOLD> make_wfrag() {
+    WFrag<N1, PAIR, FOLD> f{};
     for (int mt = 0; mt < N1 / 16; ++mt)
-        for (int kt = 0; kt < N1 / 16; ++kt)
+        for (int kt = 0; kt < f.KT; ++kt)
             for (int hl = 0; hl < 2; ++hl)
                 for (int lane = 0; lane < 32; ++lane) {
                     uint32_t r[4] = {0, 0, 0, 0};
                     for (int e = 0; e < 4; ++e) {
                         const int row = (lane >> 2) + 8 * (e & 1);
                         const int n1 = 16 * kt + 2 * (lane & 3) + 8 * (e >> 1);
-                        r[e] = half_bits(w_part(N1, row, mt, n1, hl), 0) |
-                               (half_bits(w_part(N1, row, mt, n1 + 1, hl), PAIR ? 4 : 0) << 16);
+                        r[e] = half_bits(w_part(N1, FOLD, row, mt, n1, hl), 0) |
+                               (half_bits(w_part(N1, FOLD, row, mt, n1 + 1, hl), PAIR ? 4 : 0) << 16);
                     }
                     f.v[mt][kt][hl][lane].x = r[0];
                     f.v[mt][kt][hl][lane].y = r[1];
@@ -147,20 +163,22 @@ constexpr WFrag<N1, PAIR> make_wfrag() {
     return f;
 }
 
-__device__ constexpr WFrag<16, true> kW16p = make_wfrag<16, true>();
-__device__ constexpr WFrag<32, true> kW32p = make_wfrag<32, true>();
-__device__ constexpr WFrag<32, false> kW32 = make_wfrag<32, false>();
-__device__ constexpr WFrag<64, false> kW64 = make_wfrag<64, false>();
+__device__ constexpr auto kW16p = make_wfrag<16, true, false>();
+__device__ constexpr auto kW32p = make_wfrag<32, true, false>();
+__device__ constexpr auto kW32 = make_wfrag<32, false, false>();
+__device__ constexpr auto kW32f = make_wfrag<32, false, true>();
+__device__ constexpr auto kW64f = make_wfrag<64, false, true>();
 
 template <int N1, int M>
 __device__ __forceinline__ const uint4* wfrag(int mt, int kt, int hl, int lane) {
     if constexpr (M == 1 && N1 == 16) return &kW16p.v[mt][kt][hl][lane];
     else if constexpr (M == 1) return &kW32p.v[mt][kt][hl][lane];
-    else if constexpr (N1 == 32) return &kW32.v[mt][kt][hl][lane];
-    else return &kW64.v[mt][kt][hl][lane];
+    else if constexpr (N1 == 64) return &kW64f.v[mt][kt][hl][lane];
+    else if constexpr (folded(M)) return &kW32f.v[mt][kt][hl][lane];
+    else return &kW32.v[mt][kt][hl][lane];
 }
 
-// Twiddles [mt][p][j][g]: W_K^{j (k1 + N1 p)} with k1 = 8 mt + g, as (re a, re b,
+// Twiddles [mt][p][j][g]: W_K^{j (k1 + N1 p)}, k1 of the row, as (re a, re b,
 // im a, im b) for the lane's two transforms: frames a and b, equal but in the
 // special row (m-tile 0, g = 0), whose second transform is k1 = N1/2; times
 // 2^24 (2^20 for odd j: high nibbles), half of it in the special row (the
@@ -179,8 +197,9 @@ constexpr TwTab<N1, M> make_tw() {
             for (int j = 0; j < T::MC; ++j)
                 for (int g = 0; g < 8; ++g) {
                     const bool sp = M > 1 && mt == 0 && g == 0;
-                    const int ma = j * (8 * mt + g + N1 * p);
-                    const int mb = j * ((sp ? N1 / 2 : 8 * mt + g) + N1 * p);
+                    const int k1 = k1_of(folded(M), mt, g);
+                    const int ma = j * (k1 + N1 * p);
+                    const int mb = j * ((sp ? N1 / 2 : k1) + N1 * p);
                     const double s = ((j & 1) ? 1048576.0 : 16777216.0) * (sp ? 0.5 : 1.0);
                     float4& o = f.v[mt][(p * T::MC + j) * 8 + g];
                     o.x = (float)(s * cos_k(ma, N1 * M));
@@ -227,6 +246,11 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ uint32_t pack_h2(float a, float b) {
     const __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ uint32_t sub_h2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
 }
 // The FP32 values minus the FP16 pair rounded from them (exact)
 __device__ __forceinline__ float2 minus_h2(float a, float b, uint32_t h) {
@@ -386,6 +410,8 @@ struct MmaShape {
     static constexpr int MC = M < 16 ? M : 16;       // points of the in-register DFT
     static constexpr int Q = M / MC;                 // radix step before it (M = 32: 2)
     static constexpr int TW = MTC * Q * MC * 8;      // twiddles per antenna
+    static constexpr bool kFold = folded(M);         // half the matrix columns
+    static constexpr int KT = N1 / 16 / (kFold ? 2 : 1);
     static constexpr bool kAsync = K >= 512;         // samples through shared memory
     static constexpr int kRaw = kAsync ? K / 2 : 0;  // bytes of a frame in the sample buffer
     static constexpr int row_bytes(int out) {        // a channel's Re and Im, 32 frames, one plane
@@ -402,7 +428,7 @@ struct MmaShape {
     static size_t smem(int out, bool corr, int an, int ns) {
         const size_t rows = (size_t)ROWS * an;
         return (out == kOutDebug ? 0 : 1024) + (size_t)ns * an * unit_bytes(out) +
-               kMmaFrames * kRaw + ((size_t)an * TW + MTC * (N1 / 16) * 64) * sizeof(float4) + (corr ? rows * sizeof(float4) : 0) +
+               kMmaFrames * kRaw + ((size_t)an * TW + MTC * KT * 64) * sizeof(float4) + (corr ? rows * sizeof(float4) : 0) +
                (out == SPEC_F16 || out == SPEC_F8 ? rows * sizeof(float2) : 0);
     }
 };
@@ -411,7 +437,7 @@ struct MmaShape {
 // which hold conj X[K - k], K - k (the k1 = N1/2 channels in the special row).
 template <int N1, int M>
 __device__ __forceinline__ int mma_channel(int mt, int k2, int g) {
-    const int k1 = 8 * mt + g;
+    const int k1 = k1_of(folded(M), mt, g);
     if (M == 1 || k2 < M / 2) return k1 + N1 * k2;
     return N1 * (M - k2) - (k1 == 0 ? N1 / 2 : k1);
 }
@@ -423,7 +449,7 @@ __device__ __forceinline__ int mma_channel(int mt, int k2, int g) {
 // m-tile 0 alone the conjugated half has 7 adjacent channels and the k1 = N1/2
 // one apart (part7, part1; one slot each).
 struct OutMaps {
-    CUtensorMap full, part7, part1;
+    CUtensorMap full, odd, part7, part1;
 };
 
 // Units of work: 32-frame blocks of AN antennas, all m-tiles (M < 16) or one.
@@ -438,8 +464,9 @@ __global__ void __launch_bounds__(kMmaThreads, MINB)
 fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMaps maps, int AN,
             int nfb, int64_t units) {
     using Sh = MmaShape<N1, M, MTC>;
-    constexpr int K = Sh::K, C = Sh::C, KT = N1 / 16, MC = Sh::MC, Q = Sh::Q, KB = Sh::KB;
-    constexpr int NB = 2 * KT;                         // sample pairs per lane and n2
+    constexpr int K = Sh::K, C = Sh::C, KT = Sh::KT, MC = Sh::MC, Q = Sh::Q, KB = Sh::KB;
+    constexpr int NB = N1 / 8;                         // sample pairs per lane and n2
+    constexpr bool kFold = Sh::kFold;
     constexpr bool DEBUG = OUT == kOutDebug;
     constexpr bool kScaled = OUT == SPEC_F16 || OUT == SPEC_F8;
     constexpr bool kAsync = Sh::kAsync;
@@ -543,6 +570,7 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
     };
 
     static_assert(MTC <= 2 && (MTC == 1 || MTC == N1 / 16), "m-tiles of a CTA: one, or both");
+    static_assert(kFold == (Sh::MTG > 1) && kFold == kAsync, "one m-tile per CTA: folded");
     uint4* wtab = reinterpret_cast<uint4*>(tw + AN * Sh::TW);   // [m-tile][kt][hi, lo][lane]
     for (int e = tid; e < MTC * KT * 64; e += kMmaThreads)
         wtab[e] = __ldg(wfrag<N1, M>(mt0, 0, 0, 0) + e);
@@ -588,8 +616,10 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
         bool fresh = true;                             // nothing staged in this unit yet
 
         // One m-tile of one antenna; SP: m-tile 0, whose row g = 0 is special.
-        auto unit = [&](auto sp, int ml, int ai) {
+        // ODD (folded): k1 odd.
+        auto unit = [&](auto sp, auto odd, int ml, int ai) {
                 constexpr bool SP = decltype(sp)::value;
+                [[maybe_unused]] constexpr bool ODD = decltype(odd)::value;
                 [[maybe_unused]] const int mt = SP ? 0 : mt0 + ml;
                 const bool special = SP && g == 0;
                 if constexpr (kAsync) {
@@ -627,6 +657,11 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
                             B[b] = and_xor(t, mhi, 0x00800080u);
                         else
                             B[b] = and_xor(t, mlo, 0x00080008u);
+                    }
+                    if constexpr (kFold) {             // exact: subnormals add as integers
+#pragma unroll
+                        for (int b = 0; b < NB / 2; ++b)
+                            B[b] = ODD ? sub_h2(B[b], B[b + NB / 2]) : B[b] + B[b + NB / 2];
                     }
                     float h[4], l[4];
                     mma16816(h, W[0][0], B[0], B[1], 0.f, 0.f, 0.f, 0.f);
@@ -676,7 +711,7 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
                 const float4* tm = tw + (ai * MTC + ml) * (Q * MC * 8) + g;
                 if constexpr (Q == 2) {
                     // radix 2 over n2 and n2 + 16 (p = k2 mod 2)
-                    const float2 pa = __ldg(a.twiddle + ((16 * (8 * mt + g)) & (K - 1)));
+                    const float2 pa = __ldg(a.twiddle + ((16 * k1_of(kFold, mt, g)) & (K - 1)));
                     const float2 pb = SP && special ? __ldg(a.twiddle + ((16 * (N1 / 2)) & (K - 1))) : pa;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
@@ -799,15 +834,17 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
         if constexpr (MTC == 1) {
             for (int ai = 0; ai < an; ++ai) {
                 if (mt0 == 0)
-                    unit(std::true_type{}, 0, ai);
-                else
-                    unit(std::false_type{}, 0, ai);
+                    unit(std::true_type{}, std::false_type{}, 0, ai);
+                else if (kFold && (mt0 & 1))
+                    unit(std::false_type{}, std::bool_constant<kFold>{}, 0, ai);
+                else if (!kFold || Sh::MT > 2)
+                    unit(std::false_type{}, std::false_type{}, 0, ai);
             }
         } else {
 #pragma unroll 1
-            for (int ai = 0; ai < an; ++ai) unit(std::true_type{}, 0, ai);
+            for (int ai = 0; ai < an; ++ai) unit(std::true_type{}, std::false_type{}, 0, ai);
 #pragma unroll 1
-            for (int ai = 0; ai < an; ++ai) unit(std::false_type{}, 1, ai);
+            for (int ai = 0; ai < an; ++ai) unit(std::false_type{}, std::false_type{}, 1, ai);
         }
         if constexpr (!DEBUG) {
             // the staged boxes go out by TMA, one lane of each warp issuing
@@ -822,15 +859,18 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
                     const uint32_t sm = stg + ai * kUnitB + pl * (kUnitB / kPlanes) + half * kHalfB;
                     const int row = OUT == SPEC_F16X2 || OUT == SPEC_F16 ? i0 + ai : 2 * (i0 + ai);
                     const int t = tile + pl * lo_tile;
+                    // (folded: maps of every second channel)
+                    const CUtensorMap* full = kFold && (mt0 & 1) ? &maps.odd : &maps.full;
                     if (half == 0)
-                        tc::tma_store_5d(&maps.full, sm, x, row, 8 * mt0, 0, t);
+                        tc::tma_store_5d(full, sm, x, row, kFold ? 8 * (mt0 >> 1) : 8 * mt0, 0, t);
                     else if (!split)
-                        tc::tma_store_5d(&maps.full, sm, x, row, Sh::MTG == 1 ? N1 / 2 : N1 - 7 - 8 * mt0, 0, t);
+                        tc::tma_store_5d(full, sm, x, row,
+                                         kFold ? N1 / 2 - 7 - 8 * (mt0 >> 1) - (mt0 & 1) : N1 / 2, 0, t);
                     else
                         for (int sl = 0; sl < Sh::H; ++sl) {
                             const uint32_t ss = sm + sl * Sh::split_slot(OUT);
-                            tc::tma_store_5d(&maps.part7, ss, x, row, N1 - 7, sl, t);
-                            tc::tma_store_5d(&maps.part1, ss + (OUT == SPEC_F8 ? 512 : 7 * kRowB), x, row, N1 / 2, sl, t);
+                            tc::tma_store_5d(&maps.part7, ss, x, row, N1 / 2 - 7, sl, t);
+                            tc::tma_store_5d(&maps.part1, ss + (OUT == SPEC_F8 ? 512 : 7 * kRowB), x, row, N1 / 4, sl, t);
                         }
                 }
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -860,21 +900,21 @@ cudaError_t make_maps(const FengineArgs& a, OutMaps& m) {
                                  ? 2 * (cuuint64_t)(a.plane_stride / ((int64_t)Sh::C * 2 * a.N)) / T
                                  : ((cuuint64_t)(a.s_base + a.S_pad) + T - 1) / T;
     const cuuint64_t dims[5] = {pairs ? 2 * T : T, pairs ? (cuuint64_t)a.N : 2 * (cuuint64_t)a.N,
-                                (cuuint64_t)(M > 1 ? N1 : N1 / 2), (cuuint64_t)Sh::H, tiles};
-    const cuuint64_t str[4] = {(pairs ? 2 : 1) * T * eb, rowb, N1 * rowb, Sh::C * rowb};
+                                (cuuint64_t)(M == 1 || Sh::kFold ? N1 / 2 : N1), (cuuint64_t)Sh::H, tiles};
+    const cuuint64_t str[4] = {(pairs ? 2 : 1) * T * eb, (Sh::kFold ? 2 : 1) * rowb, N1 * rowb, Sh::C * rowb};
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     const CUtensorMapDataType dt = eb == 4   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : eb == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                              : CU_TENSOR_MAP_DATA_TYPE_UINT8;
     const CUtensorMapSwizzle sw = eb == 1 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_128B;
-    auto enc = [&](CUtensorMap& t, cuuint32_t nch, cuuint32_t nsl) {
+    auto enc = [&](CUtensorMap& t, cuuint32_t nch, cuuint32_t nsl, cuuint64_t first = 0) {
         const cuuint32_t box[5] = {pairs ? 64u : 32u, pairs ? 1u : 2u, nch, nsl, 1};
-        return tc::get_encoder()(&t, dt, 5, a.spec, dims, str, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+        return tc::get_encoder()(&t, dt, 5, static_cast<char*>(a.spec) + first, dims, str, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                                  CU_TENSOR_MAP_L2_PROMOTION_NONE,
                                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     bool ok = enc(m.full, Sh::KB, Sh::H);
-    if (Sh::MTG > 1) ok = ok && enc(m.part7, 7, 1) && enc(m.part1, 1, 1);
+    if (Sh::kFold) ok = ok && enc(m.odd, Sh::KB, Sh::H, rowb) && enc(m.part7, 7, 1) && enc(m.part1, 1, 1);
     return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 
