@@ -165,6 +165,14 @@ int corr_get_scales(corr_t h, float* scales);
  * batches (corr_batch_*) reject handles with delays set (CORR_EINVAL). */
 int corr_set_sample_delays(corr_t h, const int32_t* delays);
 
+/* on: later pushes and passes of an FP32 handle round as the FP32 kernels
+ * always have (FFTs in FP32 throughout, passes cut as for single CTAs), so
+ * FP64 visibilities stay the same to the bit from one version to the next, as
+ * a loss and its finite differences want; off (the default): the fastest
+ * kernels, equally accurate.  The autograd binding turns it on for its
+ * forward pass. */
+int corr_set_stable(corr_t h, int on);
+
 /* Correlate n samples per antenna (n a multiple of K, n >= 0) and add them
  * to the running integration.  `samples` holds n/K frames in the layout
  * above (n*N/2 bytes).  Host memory is staged through the handle's pinned

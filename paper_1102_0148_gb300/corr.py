@@ -58,6 +58,7 @@ _SIGS = {
     "corr_correlate_noalloc": (_int, [_vp, _i64, _int, _int, _vp, _vp]),
     "corr_set_scales": (_int, [_vp, _vp]),
     "corr_set_sample_delays": (_int, [_vp, _vp]),
+    "corr_set_stable": (_int, [_vp, _int]),
     "corr_batch_create": (_int, [ctypes.POINTER(_vp), _int, ctypes.POINTER(_int), ctypes.POINTER(_int), _int]),
     "corr_batch_set_chunk": (_int, [_vp, _i64]),
     "corr_batch_set_tiles": (_int, [_vp, _int, _int, _int, _int]),
@@ -199,6 +200,11 @@ def corr_set_sample_delays(h, delays):
     if delays is not None and isinstance(delays, (list, tuple, np.ndarray)):
         delays = np.ascontiguousarray(np.asarray(delays, np.int32))
     return _check(_lib.corr_set_sample_delays(h, _addr(delays)), h)
+
+
+def corr_set_stable(h, on):
+    """Round as the FP32 kernels always have (on), or take the fastest ones."""
+    return _check(_lib.corr_set_stable(h, 1 if on else 0), h)
 
 
 def corr_dump_async(h, vis, fp64=False):

@@ -96,6 +96,7 @@ struct corr_s {
     int f_next = 0;
     cudaStream_t f_last = nullptr;   // stream of the latest F-engine launch
     cudaEvent_t f_span = nullptr;    // profiling: start of the open run of side launches
+    bool stable = false;      // corr_set_stable
     // coarse integer sample delays (corr_set_sample_delays)
     bool sdelay_on = false;
     int* sdelay = nullptr;          // [N] samples, device
@@ -378,6 +379,7 @@ FengineArgs fengine_args(corr_t h, const uint8_t* din, int64_t S, bool raw, int6
     fa.spec_type = h->spec_type;
     fa.scale = (h->spec_type == SPEC_F16 || h->spec_type == SPEC_F8) ? h->scale : nullptr;
     fa.split = split_table(h, raw);
+    fa.stable = h->stable;
     fa.debug_out = nullptr;
     return fa;
 }
@@ -453,6 +455,7 @@ int xengine_pass(corr_t h, int64_t S_pad, double2* acc) {
         run.scale = h->scale;
         run.split = h->fill_split;
         run.status = h->status;
+        run.stable = h->stable;
         run.assign = acc == h->acc && h->acc_zero;
         TcPlan* plans[1] = {h->tc};
         int rc = tc_launch(plans, 1, &run, h->stream, h->err);
@@ -1083,6 +1086,12 @@ int corr_test_fault(corr_t h, int kind, double wait_limit_s) {
     if (jrc != CORR_OK) return jrc;
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     return tc_test_withhold(h->tc, wait_limit_s, h->err);
+}
+
+int corr_set_stable(corr_t h, int on) {
+    if (!h) return CORR_EINVAL;
+    h->stable = on != 0;
+    return CORR_OK;
 }
 
 int corr_set_sample_delays(corr_t h, const int32_t* delays) {

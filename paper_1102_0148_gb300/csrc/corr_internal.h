@@ -100,6 +100,7 @@ struct FengineArgs {
     // Set by launch_fengine: the K = 512 grid runs antenna fastest
     // (blockIdx.x = antenna) unless its frame blocks exceed gridDim.y's limit.
     int ant_x;
+    int stable;              // FP32 and pair outputs from the FP32 kernels (corr_set_stable)
 };
 
 cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st);

@@ -756,19 +756,22 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
             default: return go2(fengine_k1024<SPEC_F16X2, false>, fengine_k1024<SPEC_F16X2, true>);
         }
     }
-    if (a.K == 4096 && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
+    // (K = 2048: stable FP32 outputs)
+    if ((a.K == 2048 || a.K == 4096) && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
         const int64_t fr = dbg ? a.S : a.S_pad;
         if (fr <= 0) return cudaSuccess;
-        using Sh = Rad16Shape<8>;
-        const size_t smem = Sh::smem(dbg);
+        const int FT = a.K == 2048 ? Rad16Shape<4>::FT : Rad16Shape<8>::FT;
+        const size_t smem = a.K == 2048 ? Rad16Shape<4>::smem(dbg) : Rad16Shape<8>::smem(dbg);
         auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem);
             if (e != cudaSuccess) return e;
-            dim3 grid((unsigned)((fr + Sh::FT - 1) / Sh::FT), (unsigned)a.N);
+            dim3 grid((unsigned)((fr + FT - 1) / FT), (unsigned)a.N);
             kern<<<grid, kRadThreads, smem, st>>>(a);
             return cudaGetLastError();
         };
+        if (a.K == 2048)
+            return a.spec_type == SPEC_F32 ? go(fengine_rad16<4, SPEC_F32>) : go(fengine_rad16<4, SPEC_F16X2>);
         if (dbg) return go(fengine_rad16<8, kOutDebug>);
         switch (a.spec_type) {
             case SPEC_F32: return go(fengine_rad16<8, SPEC_F32>);

@@ -974,6 +974,7 @@ cudaError_t launch_shape(const FengineArgs& a, cudaStream_t st) {
 
 bool fengine_mma_serves(const FengineArgs& a) {
     if (a.K < 16 || a.K > 2048) return false;
+    if (a.stable && (a.spec_type == SPEC_F32 || a.spec_type == SPEC_F16X2)) return false;
     // bytes of the widest load: one pair of n1, at least a cp.async for K >= 512
     const uintptr_t align = a.K >= 512 ? 16 : (a.K <= 32 ? 1 : a.K / 32);
     if (reinterpret_cast<uintptr_t>(a.in) % align) return false;

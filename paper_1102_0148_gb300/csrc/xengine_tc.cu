@@ -1212,9 +1212,14 @@ LaunchShape launch_shape(const TcPlan* lead, TcPlan* const* plans, int n) {
 // cut moves elsewhere unless a pass has few channels and many spectra (N =
 // 100, K = 512, 2048 frames FP16: 68 us whole, 206 cut in two; N = 192, 4096
 // frames: 245 against 470).
-DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int64_t* S_pad) {
+// stable: where a pass is cut sets how its FP32 sums round, so visibilities
+// that are to stay the same to the bit take the cuts of the deal to single
+// CTAs (one A block against two B blocks), whatever the pairs would do best.
+DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int64_t* S_pad, bool stable) {
     std::vector<int64_t> key(S_pad, S_pad + n);
     DealPlan out;
+    stable = stable && n == 1 && plans[0]->nblk > 1;
+    if (stable) key.push_back(1);
     if (lead->split > 0) {
         // fixed by corr_set_tiles: round-robin, ranges per channel, at most one per k-tile
         out.sp.resize(n);
@@ -1228,7 +1233,7 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
     for (auto& e : cache)
         if (e.first == key) return e.second;
     // workers: CTAs, or with several antenna blocks CTA pairs
-    const int sms = plans[0]->nblk > 1 ? plans[0]->num_sms / 2 : plans[0]->num_sms;
+    const int sms = plans[0]->nblk > 1 && !stable ? plans[0]->num_sms / 2 : plans[0]->num_sms;
     int64_t max_tiles = 1;
     for (int m = 0; m < n; ++m) max_tiles = std::max<int64_t>(max_tiles, S_pad[m] / plans[m]->KT);
     std::vector<int> best(n, 1);
@@ -1237,7 +1242,7 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
     // cost of an item's end and of its share in combining partials, in k-tiles
     // (FP32 mode, FP16, FP8; a group's k-tile takes 0.5, 0.2 and 0.4 us)
     static const double kGroupEnd[3] = {3, 8, 4}, kGroupCombine[3] = {70, 180, 90};
-    const bool groups = plans[0]->nblk > 1;
+    const bool groups = plans[0]->nblk > 1 && !stable;
     const double end = groups ? kGroupEnd[plans[0]->mode] : 4.0;
     const double combine = groups ? kGroupCombine[plans[0]->mode] : 2.0;
     for (int64_t T = 1; T <= max_tiles * 2; T *= 2) {
@@ -1258,6 +1263,14 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
             for (int s = 0; s < sp[m]; ++s) {
                 const int64_t t = std::min<int64_t>(per, tiles - (int64_t)s * per);
                 for (int k = 0; k < p->C; ++k) {
+                    if (stable) {
+                        // one A block against two B blocks each, a unit per tile and one
+                        for (int b1 = 0; b1 < p->nblk; ++b1)
+                            for (int b2 = b1; b2 < p->nblk; b2 += 2, ++g)
+                                load[g % sms] += (double)t * 0.5 * (std::min(2, p->nblk - b2) + (b2 != b1) + 1) +
+                                                 end + (sp[m] > 1 ? combine : 0.0);
+                        continue;
+                    }
                     const int turn = group_turn((int)g, p->npairs, sms);
                     for (int pr = 0; pr < p->npairs; ++pr, ++g)
                         load[g % sms] +=
@@ -1338,7 +1351,7 @@ int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, cu
                std::string& err) {
     std::vector<int64_t> S(n);
     for (int m = 0; m < n; ++m) S[m] = runs[m]->S_pad;
-    const DealPlan deal = choose_deal(lead, plans, n, S.data());
+    const DealPlan deal = choose_deal(lead, plans, n, S.data(), runs[0]->stable);
     const std::vector<int>& sp = deal.sp;
     const LaunchShape L = launch_shape(lead, plans, n);
     TcArgs a;
