@@ -95,8 +95,10 @@ struct corr_s {
     bool f_pending[2] = {false, false};
     int f_next = 0;
     cudaStream_t f_last = nullptr;   // stream of the latest F-engine launch
+    bool f_mma = false;              // which kind of kernel it was (fengine_mma_serves)
     cudaEvent_t f_span = nullptr;    // profiling: start of the open run of side launches
     bool stable = false;      // corr_set_stable
+    int64_t total = 0;        // frames of the integration with the push under way
     // coarse integer sample delays (corr_set_sample_delays)
     bool sdelay_on = false;
     int* sdelay = nullptr;          // [N] samples, device
@@ -379,6 +381,7 @@ FengineArgs fengine_args(corr_t h, const uint8_t* din, int64_t S, bool raw, int6
     fa.spec_type = h->spec_type;
     fa.scale = (h->spec_type == SPEC_F16 || h->spec_type == SPEC_F8) ? h->scale : nullptr;
     fa.split = split_table(h, raw);
+    fa.total = h->total;
     fa.stable = h->stable;
     fa.debug_out = nullptr;
     return fa;
@@ -398,6 +401,13 @@ int fengine_pass(corr_t h, const uint8_t* din, int64_t S, bool raw, int64_t off)
     }
     CUDA_TRY(h, cudaEventRecord(h->f_fork, h->stream));
     CUDA_TRY(h, cudaStreamWaitEvent(st, h->f_fork, 0));
+    // Launches of one kind follow each other's tails closely.  Persistent CTAs
+    // that start into the tail of the other kind stay staggered from launch to
+    // launch (an FP8 second at 35 MS/s: F-engine 1105 against 993 us), so a
+    // change of kind waits for the launch before it.
+    const bool mma = fengine_mma_serves(fa);
+    if (mma != h->f_mma && h->f_pending[j ^ 1]) CUDA_TRY(h, cudaStreamWaitEvent(st, h->f_done[j ^ 1], 0));
+    h->f_mma = mma;
     CUDA_TRY(h, launch_fengine(fa, st));
     CUDA_TRY(h, cudaEventRecord(h->f_done[j], st));
     h->f_pending[j] = true;
@@ -602,6 +612,7 @@ void free_stages(corr_t h) {
 // X-engine into `acc` whenever it fills up.
 int process_samples(corr_t h, const uint8_t* samples, int64_t n, bool raw, double2* acc) {
     const int64_t frames = n / h->K;
+    h->total = (raw ? 0 : h->n_spec) + frames;
     const int64_t rec = (int64_t)h->N * (h->K / 2);
     const bool host = !is_device_ptr(samples);
     // (the fused F-engine reads 16 bytes per lane: 16-byte aligned input only)
@@ -1494,6 +1505,7 @@ int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* 
     int64_t frames[kMaxTcModes], passes = 0;
     for (int m = 0; m < b->n; ++m) {
         frames[m] = n[m] / b->h[m]->K;
+        b->h[m]->total = b->h[m]->n_spec + frames[m];
         passes = std::max(passes, (frames[m] + b->h[m]->cap - 1) / b->h[m]->cap);
     }
     for (int64_t pi = 0; pi < passes; ++pi) {

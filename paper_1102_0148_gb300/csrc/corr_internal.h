@@ -100,6 +100,7 @@ struct FengineArgs {
     // Set by launch_fengine: the K = 512 grid runs antenna fastest
     // (blockIdx.x = antenna) unless its frame blocks exceed gridDim.y's limit.
     int ant_x;
+    int64_t total;           // frames of the integration with this push (0: S)
     int stable;              // FP32 and pair outputs from the FP32 kernels (corr_set_stable)
 };
 

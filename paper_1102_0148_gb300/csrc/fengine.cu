@@ -703,8 +703,8 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
     const bool dbg = a.debug_out != nullptr;
     if (fengine_mma_serves(a)) return launch_fengine_mma(a, st);
     // K = 512 with 16-byte aligned input (the kernel reads 16 B per lane): the
-    // FP32 and FP16-pair outputs, bound by their own bytes (350 us per 16384
-    // frames at N = 44 in FP32 mode either way)
+    // FP32 and FP16-pair outputs, bound by their own bytes (346 us per 16384
+    // frames at N = 44 in FP32 mode, 369 with the other), and short FP8 passes
     if (a.K == 512 && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
         const int64_t fr = dbg ? a.S : a.S_pad;
         if (fr <= 0) return cudaSuccess;
@@ -713,9 +713,10 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         b.ant_x = nfb <= 65535;
         const dim3 grid = b.ant_x ? dim3((unsigned)a.N, (unsigned)nfb) : dim3((unsigned)nfb, (unsigned)a.N);
         // staging (also the exchange areas), the twiddle bases, and when used
-        // the corrections, for the debug output too (at most 72 KB: three CTAs
-        // per SM)
+        // the scales and the corrections, for the debug output too (at most 72
+        // KB: three CTAs per SM)
         const size_t smem = (size_t)kStgFloats * sizeof(float) + 128 * sizeof(float2) +
+                            (!dbg && a.spec_type == SPEC_F8 ? 256 * sizeof(float) : 0) +
                             (a.corr ? 256 * sizeof(float2) : 0);
         auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -728,6 +729,7 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         if (dbg) return go2(fengine_k512<kOutDebug, false>, fengine_k512<kOutDebug, true>);
         switch (a.spec_type) {
             case SPEC_F32: return go2(fengine_k512<SPEC_F32, false>, fengine_k512<SPEC_F32, true>);
+            case SPEC_F8: return go2(fengine_k512<SPEC_F8, false>, fengine_k512<SPEC_F8, true>);
             default: return go2(fengine_k512<SPEC_F16X2, false>, fengine_k512<SPEC_F16X2, true>);
         }
     }
@@ -739,9 +741,10 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         FengineArgs b = a;
         b.ant_x = 0;
         const dim3 grid((unsigned)nfb, (unsigned)a.N);
-        // staging (also the exchange areas) and the twiddle tables, for the
-        // debug output too (at most 70 KB: three CTAs per SM)
-        const size_t smem = (size_t)kStg1024Floats * sizeof(float) + (256 + 32) * sizeof(float2);
+        // staging (also the exchange areas), the twiddle tables and for FP8 the
+        // scales, for the debug output too (at most 71 KB: three CTAs per SM)
+        const size_t smem = (size_t)kStg1024Floats * sizeof(float) + (256 + 32) * sizeof(float2) +
+                            (!dbg && a.spec_type == SPEC_F8 ? 512 * sizeof(float) : 0);
         auto go = [&](auto kern) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem);
@@ -753,10 +756,11 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
         if (dbg) return go2(fengine_k1024<kOutDebug, false>, fengine_k1024<kOutDebug, true>);
         switch (a.spec_type) {
             case SPEC_F32: return go2(fengine_k1024<SPEC_F32, false>, fengine_k1024<SPEC_F32, true>);
+            case SPEC_F8: return go2(fengine_k1024<SPEC_F8, false>, fengine_k1024<SPEC_F8, true>);
             default: return go2(fengine_k1024<SPEC_F16X2, false>, fengine_k1024<SPEC_F16X2, true>);
         }
     }
-    // (K = 2048: stable FP32 outputs)
+    // (K = 2048: stable FP32 outputs and short FP8 passes)
     if ((a.K == 2048 || a.K == 4096) && (reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
         const int64_t fr = dbg ? a.S : a.S_pad;
         if (fr <= 0) return cudaSuccess;
@@ -771,7 +775,11 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
             return cudaGetLastError();
         };
         if (a.K == 2048)
-            return a.spec_type == SPEC_F32 ? go(fengine_rad16<4, SPEC_F32>) : go(fengine_rad16<4, SPEC_F16X2>);
+            switch (a.spec_type) {
+                case SPEC_F32: return go(fengine_rad16<4, SPEC_F32>);
+                case SPEC_F8: return go(fengine_rad16<4, SPEC_F8>);
+                default: return go(fengine_rad16<4, SPEC_F16X2>);
+            }
         if (dbg) return go(fengine_rad16<8, kOutDebug>);
         switch (a.spec_type) {
             case SPEC_F32: return go(fengine_rad16<8, SPEC_F32>);

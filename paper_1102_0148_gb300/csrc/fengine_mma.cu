@@ -974,6 +974,14 @@ cudaError_t launch_shape(const FengineArgs& a, cudaStream_t st) {
 
 bool fengine_mma_serves(const FengineArgs& a) {
     if (a.K < 16 || a.K > 2048) return false;
+    // FP8 in short integrations keeps the FP32 FFTs' roundings: one E4M3
+    // rounding that falls the other way moves a visibility by up to ~0.45 of a
+    // sample's power, 0.45 / (T sqrt(2 / N + 1 / T)) of the rms visibility of T
+    // spectra.  From here on that is below 7e-4 (N = 44: T >= 3018); 1e-3 was
+    // seen at N = 44, T = 2048 and 4e-3 at N = 11, T = 120.  T: what this push
+    // brings the integration to.  FP16's roundings are 64 times finer.
+    const double T = (double)std::max(a.total, a.S);
+    if (a.spec_type == SPEC_F8 && !a.debug_out && 2.0 * T * T / a.N + T < 420000.0) return false;
     if (a.stable && (a.spec_type == SPEC_F32 || a.spec_type == SPEC_F16X2)) return false;
     // bytes of the widest load: one pair of n1, at least a cp.async for K >= 512
     const uintptr_t align = a.K >= 512 ? 16 : (a.K <= 32 ? 1 : a.K / 32);
