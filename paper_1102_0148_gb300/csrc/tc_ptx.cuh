@@ -39,39 +39,55 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// What a wait orders besides the arrivals themselves: memory written by this
+// CTA, memory written anywhere in the cluster, or nothing (tcgen05 operations
+// on either side of it are ordered by their own fences).
+enum WaitSem { kAcquireCta, kAcquireCluster, kRelaxedCluster };
+
+template <WaitSem SEM = kAcquireCta>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
+#define GBCORR_TRY_WAIT(sem)                                                              \
+    asm volatile(                                                                         \
+        "{\n\t.reg .pred p;\n\t"                                                          \
+        "mbarrier.try_wait.parity" sem ".shared::cta.b64 p, [%1], %2;\n\t"                \
+        "selp.u32 %0, 1, 0, p;\n\t}"                                                      \
+        : "=r"(ok)                                                                        \
+        : "r"(bar), "r"(parity)                                                           \
+        : "memory")
+    if (SEM == kAcquireCluster)
+        GBCORR_TRY_WAIT(".acquire.cluster");
+    else if (SEM == kRelaxedCluster)
+        GBCORR_TRY_WAIT(".relaxed.cluster");
+    else
+        GBCORR_TRY_WAIT("");
+#undef GBCORR_TRY_WAIT
     return ok != 0;
 }
 
-// Arrive at the barrier at this shared-memory offset in CTA `rank` of the
-// cluster.
-__device__ __forceinline__ void mbar_arrive_rank(uint32_t bar, uint32_t rank) {
-    asm volatile(
-        "{\n\t.reg .b32 ra;\n\t"
-        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
-        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar),
-        "r"(rank)
-        : "memory");
+// The address in CTA `rank` of the cluster of this CTA's shared-memory address.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
 }
 
-// The same with nothing of this thread's own to release: it passes on the
-// completion of TMA copies, which have landed.  (With .release.cluster, a
-// fence per stage, an FP16 pass at N = 256 took 716 us, not 589.)
-__device__ __forceinline__ void mbar_relay(uint32_t bar, uint32_t rank) {
-    asm volatile(
-        "{\n\t.reg .b32 ra;\n\t"
-        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
-        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar),
-        "r"(rank)
-        : "memory");
+// Arrive at a barrier of another CTA of the cluster (its cluster_addr), for
+// tcgen05 operations that tc_fence_before has ordered before it.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// The same, announcing `bytes` of TMA copies.  It publishes nothing else: the
+// copies' own completion on the barrier releases what they wrote.
+__device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar),
+                 "r"(bytes)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void cluster_sync() {
@@ -81,12 +97,13 @@ __device__ __forceinline__ void cluster_sync() {
 // Bounded wait on phase `parity` of `bar`.  Returns false on timeout or when
 // another role has already given up (the shared abort word is set); on
 // timeout it sets the abort word and records kStatusTimeout in `status`.
+template <WaitSem SEM = kAcquireCta>
 __device__ __forceinline__ bool wait_bar_t(uint32_t bar, uint32_t parity, volatile int* abort_word,
                                            unsigned long long timeout_ns, int* status) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<SEM>(bar, parity)) return true;
     unsigned long long t0 = 0;
     for (uint32_t n = 0;; ++n) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<SEM>(bar, parity)) return true;
         if (*abort_word) return false;
         if ((n & 63) == 63) {
             const unsigned long long now = globaltimer();
@@ -103,14 +120,23 @@ __device__ __forceinline__ bool wait_bar_t(uint32_t bar, uint32_t parity, volati
 }
 
 // Box (all frames of one k-tile, rows c1 .., channel c2, plane-and-tile c3)
-// of the tile-major workspace.
+// of the tile-major workspace.  CG 2: the barrier (a cluster_addr) may be the
+// other CTA's of the pair.
+template <int CG = 1>
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int c1, int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
+    if (CG == 1)
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(0), "r"(c1), "r"(c2), "r"(c3)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(0), "r"(c1), "r"(c2), "r"(c3)
+            : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() {

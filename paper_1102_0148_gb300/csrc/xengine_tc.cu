@@ -301,9 +301,10 @@ __device__ __forceinline__ bool next_piece(const TcArgs& a, PieceCursor& c, Piec
 }
 
 // Bounded wait with this launch's limit and status word.
+template <WaitSem SEM = kAcquireCta>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_word,
                                          const TcArgs& a) {
-    return wait_bar_t(bar, parity, abort_word, a.timeout_ns, a.status);
+    return wait_bar_t<SEM>(bar, parity, abort_word, a.timeout_ns, a.status);
 }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
@@ -341,6 +342,48 @@ __device__ __forceinline__ ItemLayout item_layout(const TcArgs& a, const TcModeA
     return L;
 }
 
+// How far a pair's CTAs came (see WIDE below); rank 0 writes most of it in both.
+struct PairEnd {
+    int loads[2];       // stage loads of each rank (in rank 0)
+    int skipped;        // rank 0's first one, left out by the test hook
+    int commits;        // stages and windows whose MMAs rank 0 committed
+    int windows;
+    int drain;          // rank 0 committed to the drain barrier
+    int abort;          // the other rank gave up
+};
+
+// Times that n uses of the stages in turn come to stage s.
+__device__ __forceinline__ int turns(int n, int s, int stages) {
+    return n > s ? (n - 1 - s) / stages + 1 : 0;
+}
+
+// One thread of each CTA of a pair, when every role of both has stopped after
+// a wait ran out: the copies that either producer started (on rank 0's full
+// barriers), and the arrivals of rank 0's commits at this CTA's barriers.
+// Waits are bounded.
+__device__ __noinline__ void pair_drain(const PairEnd& e, int rank, int stages, uint64_t* full,
+                                        uint64_t* empty, uint64_t* accf, uint64_t* drain,
+                                        unsigned long long timeout_ns) {
+    const unsigned long long until = globaltimer() + timeout_ns;
+    auto over = [&](uint64_t* bar, int phases) {      // the last of the barrier's phases
+        while (phases > 0 && !mbar_try_wait<kAcquireCluster>(smem_u32(bar), (uint32_t)(phases - 1) & 1u))
+            if (globaltimer() > until) break;
+    };
+    for (int s = 0; s < stages; ++s) {
+        if (rank == 0) {
+            // a producer is at most one load of a stage ahead of the other:
+            // arrive in that one's place
+            const int c0 = turns(e.loads[0], s, stages) - (s == 0 ? e.skipped : 0);
+            const int c1 = turns(e.loads[1], s, stages);
+            if (c0 != c1) mbar_arrive(smem_u32(&full[s]));
+            over(&full[s], max(c0, c1));
+        }
+        over(&empty[s], turns(e.commits, s, stages));
+    }
+    for (int b = 0; b < 2; ++b) over(&accf[b], turns(e.windows, b, 2));
+    over(drain, e.drain);
+}
+
 // WIDE: modes of several antenna blocks, worked on by pairs of CTAs (clusters
 // of two, tcgen05 cta_group::2).  A pair's MMA is M = 256 (each CTA's 128 A
 // rows, one antenna block), N up to 256 (half of the B rows in each CTA's
@@ -351,11 +394,16 @@ __device__ __forceinline__ ItemLayout item_layout(const TcArgs& a, const TcModeA
 // and loads 8 tiles per channel and k-tile at N = 256, not 12.  A pass of
 // 4096 spectra at N = 256, K = 1024: FP32 mode 2033 -> 1393 us, FP16 831 ->
 // 530, FP8 371 -> 275 (with the scales and the issue loop below).
-// Rank 0 issues the MMAs: its own tiles' barrier and the other CTA's, whose
-// warp 1 passes each full stage on by a remote arrival.  Commits arrive at
-// both CTAs' barriers; the epilogue warps of both free an accumulator set.
-// Each CTA loads with its own TMA into its own barriers, so each can wait for
-// its own copies if the launch gives up.
+// Rank 0 issues the MMAs.  Each CTA loads its own tiles, and both CTAs' copies
+// complete on rank 0's full barriers (the loads' .cta_group::2 form), whose
+// phases take the two producers' announcements and all the bytes: rank 0 waits,
+// with acquire at cluster scope, for what its MMAs read in both CTAs (256
+// antennas, K = 1024, 4096 spectra FP16 527 us, 130, K = 2048, 1500 spectra 337,
+// not above a relay of each full stage by a warp of the other CTA, 530 and 352,
+// which ordered nothing, nor above waits at CTA scope).  Commits arrive at both CTAs'
+// barriers; the epilogue warps of both free an accumulator set.
+// If a launch gives up, a pair's CTAs exchange how far they came and wait for
+// everything still under way to either (pair_drain) before one may end.
 template <int MODE, bool WIDE>
 __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_constant__ TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
@@ -377,6 +425,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
     const uint32_t bl_off = bh_off + slot;                          // B half: lo (planes == 2)
     const uint32_t atom_bytes = planes * slot * (WIDE ? 2u : 1u);
     constexpr bool single = !WIDE;
+    constexpr int CG = WIDE ? 2 : 1;
     const int rank = WIDE ? (int)(blockIdx.x & 1) : 0;              // CTA of the pair
     const uint32_t stage_bytes = atom_bytes * (uint32_t)a.atoms;
     unsigned char* stages = smem;
@@ -398,13 +447,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
     Piece* epi_pc = reinterpret_cast<Piece*>(epi_cur + 1);
     volatile int* epi_more = reinterpret_cast<volatile int*>(epi_pc + 2);   // [2], as epi_pc
     volatile int* epi_abort = epi_more + 2;
+    PairEnd* pair_end = reinterpret_cast<PairEnd*>(const_cast<int*>(epi_abort + 1));
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < a.stages; ++s) {
-            mbar_init(smem_u32(&full[s]), WIDE && rank == 0 ? 2 : 1);   // own copies, relay
+            mbar_init(smem_u32(&full[s]), WIDE ? 2 : 1);       // one per producer
             mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -413,6 +463,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         }
         mbar_init(smem_u32(drain), 1);
         *abort_word = 0;
+        if (WIDE) *pair_end = PairEnd{};
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -448,7 +499,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         uint32_t st = 0, ph = 0;               // stage slot and its phase parity
         uint32_t armed = 0, armed_ph = 0;      // slots with copies in flight, their parity
         bool ok = true, first = true;
+        int loads = 0;
         const uint32_t stage0 = smem_u32(stages);
+        const uint32_t full0 = WIDE ? cluster_addr(smem_u32(full), 0) : smem_u32(full);
         PieceCursor cur;
         cursor_init<WIDE>(a, cur);
         Piece pc;
@@ -472,18 +525,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 }
                 if (!(a.withhold && blockIdx.x == 0 && first)) {      // (test hook)
                     const int n_at = min(lay.at, t_end - t);
-                    const uint32_t fb = smem_u32(&full[st]);
+                    const uint32_t fb = full0 + 8u * st;
                     uint32_t dst = stage0 + st * stage_bytes;
                     if (el) {
-                        mbar_expect_tx(fb, (uint32_t)n_at * tile_bytes);
+                        if (WIDE)
+                            mbar_expect_tx_cluster(fb, (uint32_t)n_at * tile_bytes);
+                        else
+                            mbar_expect_tx(fb, (uint32_t)n_at * tile_bytes);
                         for (int at = 0; at < n_at; ++at, dst += lay.atom) {
-                            tma_load_4d(dst, map, fb, ra, itm.k, t + at);
+                            tma_load_4d<CG>(dst, map, fb, ra, itm.k, t + at);
                             if (planes == 2)
-                                tma_load_4d(dst + lay.plo, map, fb, ra, itm.k, d.cap_tiles + t + at);
+                                tma_load_4d<CG>(dst + lay.plo, map, fb, ra, itm.k, d.cap_tiles + t + at);
                             if (!alias) {
-                                tma_load_4d(dst + bh_off, map, fb, rb, itm.k, t + at);
+                                tma_load_4d<CG>(dst + bh_off, map, fb, rb, itm.k, t + at);
                                 if (planes == 2)
-                                    tma_load_4d(dst + bl_off, map, fb, rb, itm.k, d.cap_tiles + t + at);
+                                    tma_load_4d<CG>(dst + bl_off, map, fb, rb, itm.k, d.cap_tiles + t + at);
                             }
                         }
                     }
@@ -491,6 +547,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     armed_ph = (armed_ph & ~(1u << st)) | (ph << st);
                 }
                 first = false;
+                ++loads;
                 if (++st == (uint32_t)a.stages) {
                     st = 0;
                     ph ^= 1u;
@@ -504,7 +561,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 if ((armed >> s2) & 1u)
                     ok = __all_sync(0xffffffffu,
                                     wait_bar(smem_u32(&empty[s2]), (armed_ph >> s2) & 1u, abort_word, a));
-        if (!ok) {
+        if (WIDE && el) {
+            st_cluster(cluster_addr(smem_u32(&pair_end->loads[rank]), 0), loads);
+            if (a.withhold && blockIdx.x == 0) pair_end->skipped = min(loads, 1);
+        }
+        if (!WIDE && !ok) {
             // drain: every armed stage's copies must land before teardown
             const unsigned long long d2 = globaltimer() + a.timeout_ns;
             for (int s2 = 0; s2 < a.stages && s2 < 16; ++s2) {
@@ -515,38 +576,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------- MMA issuer
-        if (WIDE && rank == 1) {
-            // the pair's other CTA: pass each full stage on to rank 0
-            if (lane == 0) {
-                uint32_t st = 0, ph = 0;
-                bool ok = true;
-                PieceCursor cur;
-                cursor_init<WIDE>(a, cur);
-                Piece pc;
-                while (ok && next_piece<WIDE>(a, cur, pc)) {
-                    const TcModeArgs& d = a.md[pc.itm.m];
-                    const bool alias = pc.itm.b2 == pc.itm.b1 && group_cols(d.N, pc.itm.b2) == 256;
-                    const ItemLayout lay = item_layout(a, d, alias, planes, stage_bytes, atom_bytes, plane_off);
-                    const int t_end = (int)(pc.s_end >> a.kt_shift);
-                    for (int t = (int)(pc.s_beg >> a.kt_shift); t < t_end; t += lay.at) {
-                        ok = wait_bar(smem_u32(&full[st]), ph, abort_word, a);
-                        if (!ok) break;
-                        mbar_relay(smem_u32(&full[st]), 0);
-                        if (++st == (uint32_t)a.stages) {
-                            st = 0;
-                            ph ^= 1u;
-                        }
-                    }
-                }
-            }
-        } else {
+        // (a pair's other CTA issues none)
+        if (rank == 0) {
             const bool el = elect_one();
             uint32_t st = 0, ph = 0;
             int wi = 0;
             bool ok = true;
             bool issued = false;
+            int commits = 0, windows = 0;
+            // tiles of both CTAs are read; accumulator sets of both overwritten
+            constexpr WaitSem kFull = WIDE ? kAcquireCluster : kAcquireCta;
+            constexpr WaitSem kFree = WIDE ? kRelaxedCluster : kAcquireCta;
             const uint32_t lo0 = op_desc_lo(smem_u32(stages));
-            constexpr uint32_t CG = WIDE ? 2 : 1;
             PieceCursor cur;
             cursor_init<WIDE>(a, cur);
             Piece pc;
@@ -577,7 +618,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 for (int t = (int)(pc.s_beg >> a.kt_shift); ok && t < t_end; ++wi) {
                     const int b = wi & 1;
                     const uint32_t aph = (uint32_t)(wi >> 1) & 1u;
-                    if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&acce[b]), aph ^ 1u, abort_word, a))) {
+                    if (!__all_sync(0xffffffffu, wait_bar<kFree>(smem_u32(&acce[b]), aph ^ 1u, abort_word, a))) {
                         ok = false;
                         break;
                     }
@@ -585,7 +626,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     const int tw = min(t_end, t + wk);
                     uint32_t acc = 0;
                     for (; t < tw; t += lay.at) {
-                        if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&full[st]), ph, abort_word, a))) {
+                        if (!__all_sync(0xffffffffu, wait_bar<kFull>(smem_u32(&full[st]), ph, abort_word, a))) {
                             ok = false;
                             break;
                         }
@@ -618,6 +659,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                         }
                         acc = 1;
                         issued = true;
+                        ++commits;
+                        if (t + lay.at >= tw) ++windows;
                         if (++st == (uint32_t)a.stages) {
                             st = 0;
                             ph ^= 1u;
@@ -631,8 +674,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 const unsigned long long d2 = globaltimer() + a.timeout_ns;
                 while (!mbar_try_wait(smem_u32(drain), 0u))
                     if (globaltimer() > d2) break;
-                if (WIDE) __nanosleep(10000);      // the other CTA's arrivals of these commits
             }
+            if (WIDE && el)
+                for (int r = 0; r < 2; ++r) {
+                    st_cluster(cluster_addr(smem_u32(&pair_end->commits), r), commits);
+                    st_cluster(cluster_addr(smem_u32(&pair_end->windows), r), windows);
+                    st_cluster(cluster_addr(smem_u32(&pair_end->drain), r), !ok && issued);
+                }
         }
     } else {
         // --------------------------------------------------------- epilogue
@@ -727,7 +775,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                     if (rank == 0)
                         mbar_arrive(smem_u32(&acce[b]));
                     else
-                        mbar_arrive_rank(smem_u32(&acce[b]), 0);
+                        mbar_arrive_cluster(cluster_addr(smem_u32(&acce[b]), 0));
                 }
             }
             epi_sync();
@@ -968,10 +1016,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
     // arrive at its barriers, until here; every wait before this one is bounded)
     tc_fence_before();
     __syncwarp();
-    if (WIDE)
+    if (WIDE) {
+        if (*abort_word && lane == 0) st_cluster(cluster_addr(smem_u32(&pair_end->abort), rank ^ 1), 1);
         cluster_sync();
-    else
+        if (*abort_word || pair_end->abort) {       // the same in both CTAs
+            if (threadIdx.x == 0)
+                pair_drain(*pair_end, rank, a.stages, full, empty, accf, drain, a.timeout_ns);
+            __syncwarp();
+            cluster_sync();
+        }
+    } else {
         __syncthreads();
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
