@@ -252,6 +252,12 @@ int zero_acc(corr_t h) {
     return CORR_OK;
 }
 
+// The accumulator counts as zeros, whatever sums its memory holds.
+void acc_dumped(corr_t h) {
+    h->acc_zero = h->acc_stale = true;
+    h->part_pending = false;
+}
+
 // Wait for the handle's stream and report device-side errors.
 int wait_and_check(corr_t h) {
     int rc = queue_status(h);
@@ -1734,6 +1740,7 @@ int corr_batch_replay(corr_batch_t b, int64_t* n_spec) {
     cudaError_t e = cudaGraphLaunch(b->exec, b->stream);
     if (e != cudaSuccess)
         return batch_err(b, CORR_ECUDA, (std::string("graph launch: ") + cudaGetErrorString(e)).c_str());
+    for (int m = 0; m < b->n; ++m) acc_dumped(b->h[m]);   // the recorded dump ran, with its sums left behind
     for (int m = 0; n_spec && m < b->n; ++m) n_spec[m] = b->graph_frames[m];
     return CORR_OK;
 }
