@@ -272,7 +272,9 @@ int corr_load_state(corr_t h, const void* buf);
  * records its status); the F-engine warps stop at their next task.  The kernel then records a status
  * word, drains its own copies, frees its tensor memory and returns; the
  * next corr_dump / corr_sync reports CORR_ETIMEOUT and the handle stays
- * usable.  No GPU fault, trap or hang is involved. */
+ * usable.  No GPU fault, trap or hang is involved.
+ * kind 3 (a mode of a batch; no limit): the next corr_batch_capture fails
+ * with CORR_ECUDA, on the host, where it would record this mode's dump. */
 int corr_test_fault(corr_t h, int kind, double wait_limit_s);
 
 /* Kernel classes reported by corr_profile_read. */

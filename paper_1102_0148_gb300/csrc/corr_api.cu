@@ -122,6 +122,7 @@ struct corr_s {
     // zeros: a dump reads the slot directly, anything else that needs acc or
     // the partials first reduces it into acc (settle_partial)
     bool part_pending = false;
+    bool fail_record = false;    // test hook: the next capture fails at this handle's dump
     int64_t fill = 0;            // frames waiting in the workspace for the X-engine
     double2* fill_acc = nullptr; // accumulator those frames belong to
     TcPlan* tc = nullptr;
@@ -1097,6 +1098,10 @@ int corr_test_fault(corr_t h, int kind, double wait_limit_s) {
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
         return fx_test_withhold(h->fx, wait_limit_s, h->err);
     }
+    if (kind == 3) {
+        h->fail_record = true;
+        return CORR_OK;
+    }
     if (kind != 1) return set_err(h, CORR_EINVAL, "unknown fault kind %d", kind);
     if (!h->use_tc) return set_err(h, CORR_EINVAL, "the withheld-copy fault needs a tensor-core handle");
     int jrc = sync_fengines(h);
@@ -1697,7 +1702,9 @@ int corr_batch_capture(corr_batch_t b, const uint8_t* const* samples, const int6
         rc = batch_enqueue(b, samples, n);
         for (int m = 0; rc == CORR_OK && m < b->n; ++m) {
             corr_t h = b->h[m];
-            e = dump_ops(h, vis[m], vis_fp64, narrow(h) && !h->scales_user, b->stream, true);
+            e = h->fail_record ? cudaErrorStreamCaptureInvalidated
+                               : dump_ops(h, vis[m], vis_fp64, narrow(h) && !h->scales_user, b->stream, true);
+            h->fail_record = false;
             if (e != cudaSuccess) rc = CORR_ECUDA;
         }
         cudaGraph_t g = nullptr;
@@ -1722,6 +1729,11 @@ int corr_batch_capture(corr_batch_t b, const uint8_t* const* samples, const int6
     if (rc != CORR_OK) {
         cudaGetLastError();
         batch_free_graph(b);
+        // what was recorded never runs: each mode is as the eager dump left it
+        for (int m = 0; m < b->n; ++m) {
+            acc_dumped(b->h[m]);
+            b->h[m]->f_pending[0] = b->h[m]->f_pending[1] = false;
+        }
         if (rc == CORR_ECUDA)
             return batch_err(b, rc, (std::string("graph capture: ") + cudaGetErrorString(e)).c_str());
         return rc;

@@ -77,3 +77,24 @@ def test_empty_dumps_around_replays(lib, step):
         assert all(bool((v == f).all()) for v, f in zip(vis, first))
         _empty(b)
     _push_equals(b, B, want)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_failed_capture_leaves_no_sums(lib, step, mode):
+    """Recording fails at one mode's dump, with the passes recorded and never
+    run: every mode is as the eager step's dump left it."""
+    b, vis, B, want = step
+    lib.corr_test_fault(b.handles[mode], 3, 0.05)
+    with pytest.raises(lib.CorrError) as ei:
+        b.capture(B, vis, fp64=True)
+    assert ei.value.code == lib.CORR_ECUDA
+    with pytest.raises(lib.CorrError) as ei:
+        b.replay()
+    assert ei.value.code == lib.CORR_ESTATE
+    _push_equals(b, B, want)
+    _empty(b)
+    b.capture(B, vis, fp64=True)
+    for v in vis:
+        v.zero_()
+    _replay(b)
+    assert all(np.array_equal(v.cpu().numpy(), w) for v, w in zip(vis, want))
