@@ -176,6 +176,15 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+bool is_pageable(const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return at.type == cudaMemoryTypeUnregistered;
+}
+
 int spec_type_for(int dtype) {
     if (dtype == CORR_FP16) return SPEC_F16;
     if (dtype == CORR_FP8E4M3) return SPEC_F8;
@@ -1139,16 +1148,24 @@ int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
     if (!h) return CORR_EINVAL;
     // Host copies in page-locked memory, to check the values, to derive the
     // two-plane pre-scales and to upload from: one wait for both inputs, none
-    // for the uploads.  (The copies go through the legacy default stream, whose
-    // ordering a blocking cudaMemcpy has.)
+    // for the uploads.  The inputs may be made by work queued on the handle's
+    // stream, where the copies go, or on the legacy default stream, which they
+    // follow.  (Pageable memory is read at once.)
     CUDA_TRY(h, cudaEventSynchronize(h->corr_pin_free));   // the previous call's uploads
     float* gh = h->corr_pin;
     float* th = gh + 2 * (size_t)h->N;
-    if (gains)
-        CUDA_TRY(h, cudaMemcpyAsync(gh, gains, (size_t)h->N * sizeof(float2), cudaMemcpyDefault, 0));
-    if (delays)
-        CUDA_TRY(h, cudaMemcpyAsync(th, delays, (size_t)h->N * sizeof(float), cudaMemcpyDefault, 0));
-    if (gains || delays) CUDA_TRY(h, cudaStreamSynchronize(0));
+    const bool gp = gains && is_pageable(gains), tp = delays && is_pageable(delays);
+    if (gp) memcpy(gh, gains, (size_t)h->N * sizeof(float2));
+    if (tp) memcpy(th, delays, (size_t)h->N * sizeof(float));
+    if ((gains && !gp) || (delays && !tp)) {
+        CUDA_TRY(h, cudaEventRecord(h->corr_pin_free, cudaStreamLegacy));
+        CUDA_TRY(h, cudaStreamWaitEvent(h->stream, h->corr_pin_free, 0));
+        if (gains && !gp)
+            CUDA_TRY(h, cudaMemcpyAsync(gh, gains, (size_t)h->N * sizeof(float2), cudaMemcpyDefault, h->stream));
+        if (delays && !tp)
+            CUDA_TRY(h, cudaMemcpyAsync(th, delays, (size_t)h->N * sizeof(float), cudaMemcpyDefault, h->stream));
+        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    }
     if (gains)
         for (int i = 0; i < h->N; ++i) {
             const double a = std::hypot((double)gh[2 * i], (double)gh[2 * i + 1]);
