@@ -99,9 +99,10 @@ int corr_create(corr_t* out, int N, int K, int dtype);
 
 /* Queue later work on `stream` (a cudaStream_t of the handle's device; NULL
  * means the legacy default stream).  Waits for the handle's queued work
- * first (when the stream is the handle's already, nothing changes and there
- * is nothing to wait for). */
+ * first, also when the stream is the handle's already.
+ * corr_get_stream: the stream the handle's work is queued on. */
 int corr_set_stream(corr_t h, void* stream);
+int corr_get_stream(corr_t h, void** stream);
 
 /* Capacity of the spectra workspace in frames, rounded up to a multiple of
  * 128; default 8192 (halved while the workspace would exceed 2 GiB, not below

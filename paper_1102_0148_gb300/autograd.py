@@ -17,6 +17,14 @@ import torch
 from . import corr
 
 
+def _use_current_stream(c):
+    """Queue the handle's work on torch's current stream (switching streams
+    waits for the work queued before; staying on one needs no wait)."""
+    s = torch.cuda.current_stream().cuda_stream
+    if corr.corr_get_stream(c.h) != s:
+        corr.corr_set_stream(c.h, s)
+
+
 class Visibilities(torch.autograd.Function):
     @staticmethod
     def forward(ctx, gains, delays, samples, correlator):
@@ -25,7 +33,7 @@ class Visibilities(torch.autograd.Function):
         t = delays.detach().to(torch.float32).contiguous()
         if not (g.is_cuda and t.is_cuda and samples.is_cuda):
             raise ValueError("gains, delays and samples must be CUDA tensors")
-        corr.corr_set_stream(c.h, torch.cuda.current_stream().cuda_stream)
+        _use_current_stream(c)
         corr.corr_set_corrections(c.h, g, t)
         n = samples.numel() * 2 // c.N
         V = torch.empty((c.P, c.C), dtype=torch.complex128, device=samples.device)
@@ -47,7 +55,7 @@ class Visibilities(torch.autograd.Function):
         gV = grad_V.to(torch.complex128).contiguous()
         gg = torch.empty_like(g)
         gt = torch.empty_like(t)
-        corr.corr_set_stream(ctx.c.h, torch.cuda.current_stream().cuda_stream)
+        _use_current_stream(ctx.c)
         corr.corr_grad(ctx.c.h, samples, ctx.n, g, t, gV, True, gg, gt)
         return gg.to(ctx.dtypes[0]), gt.to(ctx.dtypes[1]), None, None
 

@@ -36,6 +36,7 @@ _int = ctypes.c_int
 _SIGS = {
     "corr_create": (_int, [ctypes.POINTER(_vp), _int, _int, _int]),
     "corr_set_stream": (_int, [_vp, _vp]),
+    "corr_get_stream": (_int, [_vp, ctypes.POINTER(_vp)]),
     "corr_set_chunk": (_int, [_vp, _i64]),
     "corr_set_tiles": (_int, [_vp, _int, _int, _int, _int]),
     "corr_set_fused": (_int, [_vp, _int]),
@@ -128,6 +129,13 @@ def corr_create(N, K, dtype=CORR_FP32):
 def corr_set_stream(h, stream):
     s = stream if isinstance(stream, int) or stream is None else stream.cuda_stream
     return _check(_lib.corr_set_stream(h, s), h)
+
+
+def corr_get_stream(h):
+    """The stream the handle's work is queued on (0: the legacy default stream)."""
+    s = _vp()
+    _check(_lib.corr_get_stream(h, ctypes.byref(s)), h)
+    return s.value or 0
 
 
 def corr_set_chunk(h, max_spectra):

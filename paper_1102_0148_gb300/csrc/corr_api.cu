@@ -900,17 +900,23 @@ int corr_create(corr_t* out, int N, int K, int dtype) {
 
 int corr_set_stream(corr_t h, void* stream) {
     if (!h) return CORR_EINVAL;
-    if (!h->own_stream && h->stream == static_cast<cudaStream_t>(stream)) return CORR_OK;
     int frc = fx_flush(h);
     if (frc != CORR_OK) return frc;
     int jrc = join_fengines(h);
     if (jrc != CORR_OK) return jrc;
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    if (h->stream == static_cast<cudaStream_t>(stream)) return CORR_OK;
     if (h->own_stream) {
         cudaStreamDestroy(h->stream);
         h->own_stream = false;
     }
     h->stream = static_cast<cudaStream_t>(stream);
+    return CORR_OK;
+}
+
+int corr_get_stream(corr_t h, void** stream) {
+    if (!h || !stream) return CORR_EINVAL;
+    *stream = h->stream;
     return CORR_OK;
 }
 
