@@ -119,8 +119,8 @@ int corr_set_chunk(corr_t h, int64_t max_spectra);
  * (1024 above 64 antennas), 2048 for FP8), `stages` = depth of the shared-memory
  * operand ring (2..16, clipped to what shared memory holds; 0 = automatic),
  * `split` = ranges of spectra per channel and antenna-block pair into which
- * a pass is cut (1..64, partials combined in a fixed order inside the
- * launch; 0 = chosen by the planner), `atoms` = k-tiles (32 spectra, 128 for
+ * a pass is cut (1..64, partials combined in a fixed order, in FP64; 0 =
+ * chosen by the planner), `atoms` = k-tiles (32 spectra, 128 for
  * FP8) carried by one pipeline stage (1..8; 0 = as many as leave three
  * stages, up to 256 spectra).  The window is rounded up to whole stages.  CORR_EINVAL for
  * CUDA-core handles or out-of-range values. */
@@ -167,7 +167,7 @@ int corr_get_scales(corr_t h, float* scales);
 int corr_set_sample_delays(corr_t h, const int32_t* delays);
 
 /* on: later pushes and passes of an FP32 handle round as the FP32 kernels
- * always have (FFTs in FP32 throughout, passes cut as for single CTAs), so
+ * always have (FFTs in FP32 throughout), so
  * FP64 visibilities stay the same to the bit from one version to the next, as
  * a loss and its finite differences want; off (the default): the fastest
  * kernels, equally accurate.  The autograd binding turns it on for its

@@ -452,19 +452,18 @@ int finish_tc_run(corr_t h, const TcRun& run, double2* acc) {
         if (acc == h->acc) h->acc_zero = h->acc_stale = false;
         return CORR_OK;
     }
-    // a multi-block mode's pass result covers every (k, p) in slot 0: the
-    // first pass of an integration stays there until a dump reads it or
-    // settle_partial stores it; later passes are added
-    if (acc == h->acc && h->acc_zero && run.n_split == 1) {
-        h->part_pending = true;
-        return CORR_OK;
+    // a multi-block mode's ranges cover every (k, p), one slot each.  The first
+    // pass of an integration is combined into slot 0 and stays there until a
+    // dump reads it or settle_partial stores it; later passes are added
+    const int64_t CP = (int64_t)h->C * h->P;
+    const bool first = acc == h->acc && h->acc_zero;
+    if (acc == h->acc && !first) h->acc_zero = h->acc_stale = false;
+    if (!first || run.n_split > 1) {
+        prof_begin(h);
+        CUDA_TRY(h, launch_combine_ranges(h->partial, run.n_split, CP, first ? nullptr : acc, h->stream));
+        prof_end(h, CORR_KERNEL_REDUCE);
     }
-    const bool assign = acc == h->acc && h->acc_zero;
-    if (acc == h->acc) h->acc_zero = h->acc_stale = false;
-    prof_begin(h);
-    CUDA_TRY(h, launch_reduce_partials(h->partial, run.n_split, (int64_t)h->C * h->P, acc,
-                                       h->stream, assign));
-    prof_end(h, CORR_KERNEL_REDUCE);
+    if (first) h->part_pending = true;
     return CORR_OK;
 }
 
@@ -481,7 +480,6 @@ int xengine_pass(corr_t h, int64_t S_pad, double2* acc) {
         run.scale = h->scale;
         run.split = h->fill_split;
         run.status = h->status;
-        run.stable = h->stable;
         run.assign = acc == h->acc && h->acc_zero;
         TcPlan* plans[1] = {h->tc};
         int rc = tc_launch(plans, 1, &run, h->stream, h->err);

@@ -148,6 +148,11 @@ cudaError_t launch_xengine_simt(XengineArgs& a, cudaStream_t st);
 cudaError_t launch_reduce_partials(const float2* partial, int n_split, int64_t CP,
                                    double2* acc, cudaStream_t st, bool assign = false);
 
+// The ranges of a multi-block pass, one per slot, summed in FP64 in slot order
+// and rounded to FP32 as a pass of one range is: added to acc, or (acc ==
+// nullptr) stored in slot 0.
+cudaError_t launch_combine_ranges(float2* partial, int n_split, int64_t CP, double2* acc, cudaStream_t st);
+
 // vis[p][k] = acc[k][p] as complex64 (fp64 == 0) or complex128.
 // scale != nullptr: also the pre-cast scales of the next integration from the
 // autocorrelations over n_spec spectra ([N][C], see scales.cuh).

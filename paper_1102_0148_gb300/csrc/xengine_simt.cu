@@ -210,6 +210,77 @@ __global__ void reduce_partials_kernel(const float2* part, int n_split, int64_t 
     }
 }
 
+// s + v = s' + e exactly (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum(float& s, float v, float& e) {
+    const float t = __fadd_rn(s, v);
+    const float b = __fsub_rn(t, s);
+    e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b));
+    s = t;
+}
+// The sum of up to 8 values, held as s + e + f to ~70 bits: rounded to FP32 it
+// is their FP64 sum rounded to FP32 (of two values: s itself), without FP64
+// conversions, which set the pace here.
+struct Sum3 {
+    float s = 0.f, e = 0.f, f = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        float t, u;
+        two_sum(s, v, t);
+        two_sum(e, t, u);
+        f = __fadd_rn(f, u);
+    }
+    __device__ __forceinline__ float value() const {
+        float h = s, t;
+        two_sum(h, e, t);
+        return __fadd_rn(h, __fadd_rn(t, f));
+    }
+};
+
+// A thread sums two pairs (C is even, so a slot is a whole number of them).
+// (The X-engine's last worker of an item combined them before, ~36 us an item
+// in FP64 on one SM while the others went idle.)
+__global__ void __launch_bounds__(256) combine_ranges_kernel(float4* part, int n_split, int64_t CP2, double2* acc) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < CP2;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        float4 r;
+        if (n_split <= 2) {
+            r = part[e];
+            if (n_split == 2) {
+                const float4 v = part[CP2 + e];
+                r = make_float4(r.x + v.x, r.y + v.y, r.z + v.z, r.w + v.w);
+            }
+        } else {
+            Sum3 t[4];
+#pragma unroll 4
+            for (int s = 0; s < n_split; ++s) {
+                const float4 v = part[(int64_t)s * CP2 + e];
+                t[0].add(v.x);
+                t[1].add(v.y);
+                t[2].add(v.z);
+                t[3].add(v.w);
+            }
+            r = make_float4(t[0].value(), t[1].value(), t[2].value(), t[3].value());
+        }
+        if (!isfinite(r.x) || !isfinite(r.y) || !isfinite(r.z) || !isfinite(r.w)) {
+            double q[4] = {0.0, 0.0, 0.0, 0.0};         // past FP32's range on the way, or NaN
+            for (int s = 0; s < n_split; ++s) {
+                const float4 v = part[(int64_t)s * CP2 + e];
+                q[0] += (double)v.x;
+                q[1] += (double)v.y;
+                q[2] += (double)v.z;
+                q[3] += (double)v.w;
+            }
+            r = make_float4((float)q[0], (float)q[1], (float)q[2], (float)q[3]);
+        }
+        if (!acc) {
+            part[e] = r;
+        } else {
+            const double2 o0 = acc[2 * e], o1 = acc[2 * e + 1];
+            acc[2 * e] = make_double2(o0.x + (double)r.x, o0.y + (double)r.y);
+            acc[2 * e + 1] = make_double2(o1.x + (double)r.z, o1.y + (double)r.w);
+        }
+    }
+}
+
 // acc [C][P] -> vis [P][C] through 32 x 32 shared-memory tiles, so both the
 // reads (along p) and the writes (along k) are coalesced.  (acc keeps its
 // sums: the next pass stores over them.)  T = double2 for the FP64
@@ -332,6 +403,11 @@ cudaError_t launch_xengine_simt(XengineArgs& a, cudaStream_t st) {
 cudaError_t launch_reduce_partials(const float2* partial, int n_split, int64_t CP, double2* acc,
                                    cudaStream_t st, bool assign) {
     reduce_partials_kernel<<<grid_for(CP), 256, 0, st>>>(partial, n_split, CP, acc, assign ? 1 : 0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_combine_ranges(float2* partial, int n_split, int64_t CP, double2* acc, cudaStream_t st) {
+    combine_ranges_kernel<<<grid_for(CP / 2), 256, 0, st>>>(reinterpret_cast<float4*>(partial), n_split, CP / 2, acc);
     return cudaGetLastError();
 }
 

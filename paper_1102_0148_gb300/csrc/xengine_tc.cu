@@ -86,7 +86,7 @@ struct TcModeArgs {
     int64_t unit_base;        // first work unit of this mode (balanced deal)
     float2* partial;          // [n_split][C][P] FP32 partials (n_split > 1)
     double2* acc;             // [C][P] FP64 accumulator
-    int* ticket;              // [C][npairs][CTAs of a worker] arrival counters (n_split > 1), zero between launches
+    int* ticket;              // [C] arrival counters of a single block (n_split > 1), zero between launches
     const float* scale;       // [N][C] pre-cast scales (modes 1, 2)
     const float* split;       // [N] two-plane pre-scales sigma_i (mode 0)
     int assign;               // acc is known to hold zeros: store instead of adding
@@ -928,13 +928,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 }
             }
             }
-            if (!direct) {
-                // The last of the CTAs sharing this (channel, block pair) to
-                // finish adds every partial, in slot order, into the FP64
-                // accumulator (a group: into slot 0, see the run's reduction):
-                // deterministic.
-                // (The two CTAs of a pair hold different rows: a counter each.)
-                int* const ticket = d.ticket + (itm.k * d.npairs + itm.pr) * (WIDE ? 2 : 1) + rank;
+            if (single && !direct) {
+                // The last of the CTAs sharing this channel to finish adds
+                // every partial, in slot order, into the FP64 accumulator:
+                // deterministic.  (A group's slots are combined by a launch of
+                // their own, launch_combine_ranges.)
+                int* const ticket = d.ticket + itm.k;
                 __threadfence();
                 epi_sync();
                 if (et == 0) {
@@ -944,11 +943,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                 epi_sync();
                 if (*epi_last) {
                     __threadfence();
-                    // every pair of the item: the single block's upper
-                    // triangle, or a group's nb1 x (64 per B block) rows and
-                    // columns (the diagonal block's upper triangle); four pairs
-                    // per thread at a time, their loads in flight together
-                    const int npl_all = single ? nb1 * (nb1 + 1) / 2 : nb1 * 64 * itm.nbB;
+                    // four pairs per thread at a time, their loads in flight together
+                    const int npl_all = nb1 * (nb1 + 1) / 2;
                     constexpr int kCB = 4;
                     for (int base = et; base < npl_all; base += kCB * 256) {
                         int pp[kCB];
@@ -956,21 +952,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
 #pragma unroll
                         for (int u = 0; u < kCB; ++u) {
                             const int pl = base + 256 * u;
-                            pp[u] = -1;
+                            pp[u] = pl < npl_all ? pl : -1;
                             re[u] = im[u] = 0.0;
-                            if (pl >= npl_all) continue;
-                            if (single) {
-                                pp[u] = pl;
-                            } else {
-                                const int i_loc = pl / (64 * itm.nbB);
-                                const int rest = pl - i_loc * 64 * itm.nbB;
-                                const int b2 = itm.b2 + (rest >> 6);
-                                const int j_loc = rest & 63;
-                                const int i = 64 * (itm.b1 + rank) + i_loc;
-                                const int j = 64 * b2 + j_loc;
-                                if (j_loc >= block_ants(N, b2) || j < i) continue;
-                                pp[u] = i * N - i * (i - 1) / 2 + (j - i);
-                            }
                         }
                         for (int sp = 0; sp < pc.nslots; ++sp) {
                             float2 v[kCB];
@@ -984,26 +967,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) xengine_tc_kernel(const __grid_
                                 im[u] += (double)v[u].y;
                             }
                         }
-                        if (single) {
-                            double2 old[kCB];
+                        double2 old[kCB];
 #pragma unroll
-                            for (int u = 0; u < kCB; ++u) {
-                                old[u] = make_double2(0.0, 0.0);
-                                if (pp[u] >= 0 && !d.assign) old[u] = d.acc[(int64_t)itm.k * P + pp[u]];
-                            }
-#pragma unroll
-                            for (int u = 0; u < kCB; ++u)
-                                if (pp[u] >= 0)
-                                    d.acc[(int64_t)itm.k * P + pp[u]] =
-                                        make_double2(old[u].x + re[u], old[u].y + im[u]);
-                        } else {
-                            // a group's pass result lives in slot 0 until the
-                            // reduction launch adds it to the accumulator
-#pragma unroll
-                            for (int u = 0; u < kCB; ++u)
-                                if (pp[u] >= 0)
-                                    d.partial[(int64_t)itm.k * P + pp[u]] = make_float2((float)re[u], (float)im[u]);
+                        for (int u = 0; u < kCB; ++u) {
+                            old[u] = make_double2(0.0, 0.0);
+                            if (pp[u] >= 0 && !d.assign) old[u] = d.acc[(int64_t)itm.k * P + pp[u]];
                         }
+#pragma unroll
+                        for (int u = 0; u < kCB; ++u)
+                            if (pp[u] >= 0)
+                                d.acc[(int64_t)itm.k * P + pp[u]] =
+                                    make_double2(old[u].x + re[u], old[u].y + im[u]);
                     }
                     if (et == 0) *ticket = 0;
                 }
@@ -1048,6 +1022,12 @@ constexpr size_t kSmemBudget = 227 * 1024;
 
 }  // namespace
 
+// Ranges per item of each mode of a step, and the busiest worker's load.
+struct RangePlan {
+    std::vector<int> sp;
+    double score = 0;
+};
+
 // How a launch deals its work to the CTAs (see next_piece).
 struct DealPlan {
     std::vector<int> sp;      // round-robin deal: ranges per item of each mode
@@ -1073,10 +1053,12 @@ struct TcPlan {
     unsigned long long timeout_ns = 4000000000ull;
     int withhold = 0;                    // test hook for the next launch
     unsigned long long hook_timeout_ns = 0;
-    int* ticket = nullptr;               // [C][npairs][2 if nblk > 1] arrival counters
-    size_t ticket_bytes() const { return (size_t)C * npairs * (nblk > 1 ? 2 : 1) * sizeof(int); }
-    // split decisions already made, keyed by the S_pad of every mode in the launch
-    std::vector<std::pair<std::vector<int64_t>, DealPlan>> split_cache;
+    int* ticket = nullptr;               // [C] arrival counters
+    size_t ticket_bytes() const { return (size_t)C * sizeof(int); }
+    // decisions already made: ranges, keyed by every mode of the step, and the
+    // deal of this plan alone, by its S_pad
+    std::vector<std::pair<std::vector<int64_t>, RangePlan>> range_cache;
+    std::vector<std::pair<int64_t, DealPlan>> deal_cache;
 };
 
 int tc_plan_create(TcPlan** out, int N, int C, int spec_type, std::string& err) {
@@ -1151,7 +1133,8 @@ int tc_plan_update(TcPlan* p, void* spec, int64_t cap, int N, int C, int spec_ty
     p->have_map = true;
     p->cap = cap;
     p->max_split = (int)std::min<int64_t>(8, (cap + 255) / 256);
-    p->split_cache.clear();
+    p->range_cache.clear();
+    p->deal_cache.clear();
     return CORR_OK;
 }
 
@@ -1176,7 +1159,8 @@ int tc_set_tiles(TcPlan* p, int window, int stages, int split, int atoms, std::s
     p->stages = stages;
     p->split = split;
     p->atoms = atoms;
-    p->split_cache.clear();
+    p->range_cache.clear();
+    p->deal_cache.clear();
     return CORR_OK;
 }
 
@@ -1254,53 +1238,29 @@ LaunchShape launch_shape(const TcPlan* lead, TcPlan* const* plans, int n) {
     return L;
 }
 
-// Work deal of one launch.  Round-robin: every mode's pass of S_pad frames
-// is cut into n_split ranges of whole k-tiles per item and items go to the
-// workers in turn; the range count minimises the busiest worker's work in a
-// simulation of that deal.  Balanced (one single-block mode): contiguous
-// shares of the weighted k-tiles (see next_piece).  The cheaper of the two in
-// the same cost model is taken: per item or piece of a single block its
-// k-tiles, ~4 more for its end, and 2 more when its partial is combined with
-// others.  At N = 44, K = 512 and 8192 frames per pass the round-robin deal
-// leaves 104 CTAs with two channels and 48 with one; the balanced deal gives
-// each 1.7 channels.  Groups: an end takes ~1.5 us, but combining the 8192
-// baselines of a CTA's tile in FP64 ~36 us, far more than the k-tiles that a
-// cut moves elsewhere unless a pass has few channels and many spectra (N =
-// 100, K = 512, 2048 frames FP16: 68 us whole, 206 cut in two; N = 192, 4096
-// frames: 245 against 470).
-// stable: where a pass is cut sets how its FP32 sums round, so visibilities
-// that are to stay the same to the bit take the cuts of the deal to single
-// CTAs (one A block against two B blocks), whatever the pairs would do best.
-DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int64_t* S_pad, bool stable) {
-    std::vector<int64_t> key(S_pad, S_pad + n);
-    DealPlan out;
-    stable = stable && n == 1 && plans[0]->nblk > 1;
-    if (stable) key.push_back(1);
-    if (lead->split > 0) {
-        // fixed by corr_set_tiles: round-robin, ranges per channel, at most one per k-tile
-        out.sp.resize(n);
-        for (int m = 0; m < n; ++m) {
-            const int64_t tiles = std::max<int64_t>(1, S_pad[m] / plans[m]->KT);
-            out.sp[m] = (int)std::min<int64_t>(std::min(lead->split, plans[m]->max_split), tiles);
-        }
-        return out;
-    }
-    auto& cache = plans[0]->split_cache;
+// Ranges into which the passes of n modes are cut, S_pad frames each: the
+// counts that minimise the busiest of the SMs in a simulated round-robin deal
+// of every mode's items to single CTAs, in units of a k-tile: the tiles, 4
+// more for an item's end and 2 when its partial is combined with others.  (A
+// group counts there as one A block against two B blocks each, one unit per
+// tile loaded and one.)  Ranges are summed in FP32 and combined in FP64, so
+// their number also bounds the rounding of a pass, for every deal below: CTA
+// pairs would gain by fewer cuts only where a pass is short (100 antennas, K =
+// 512, 2048 spectra FP16 60 us whole, 79 and 8 to combine in two; 128, 4096
+// spectra FP32 mode 268 against 244 and 11; 200, K = 16, 30000 spectra FP32
+// mode 244 against 154 and 10).
+RangePlan pass_ranges(TcPlan* const* plans, int n, const int64_t* S_pad) {
+    std::vector<int64_t> key;
+    for (int m = 0; m < n; ++m) key.insert(key.end(), {S_pad[m], plans[m]->N, plans[m]->C, plans[m]->max_split});
+    auto& cache = plans[0]->range_cache;
     for (auto& e : cache)
         if (e.first == key) return e.second;
-    // workers: CTAs, or with several antenna blocks CTA pairs
-    const int sms = plans[0]->nblk > 1 && !stable ? plans[0]->num_sms / 2 : plans[0]->num_sms;
+    const int sms = plans[0]->num_sms;
     int64_t max_tiles = 1;
     for (int m = 0; m < n; ++m) max_tiles = std::max<int64_t>(max_tiles, S_pad[m] / plans[m]->KT);
     std::vector<int> best(n, 1);
     double best_score = 1e300;
     std::vector<double> load(sms);
-    // cost of an item's end and of its share in combining partials, in k-tiles
-    // (FP32 mode, FP16, FP8; a group's k-tile takes 0.5, 0.2 and 0.4 us)
-    static const double kGroupEnd[3] = {3, 8, 4}, kGroupCombine[3] = {70, 180, 90};
-    const bool groups = plans[0]->nblk > 1 && !stable;
-    const double end = groups ? kGroupEnd[plans[0]->mode] : 4.0;
-    const double combine = groups ? kGroupCombine[plans[0]->mode] : 2.0;
     for (int64_t T = 1; T <= max_tiles * 2; T *= 2) {
         std::vector<int> sp(n);
         for (int m = 0; m < n; ++m) {
@@ -1318,21 +1278,12 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
             const int64_t per = (tiles + sp[m] - 1) / sp[m];
             for (int s = 0; s < sp[m]; ++s) {
                 const int64_t t = std::min<int64_t>(per, tiles - (int64_t)s * per);
-                for (int k = 0; k < p->C; ++k) {
-                    if (stable) {
-                        // one A block against two B blocks each, a unit per tile and one
-                        for (int b1 = 0; b1 < p->nblk; ++b1)
-                            for (int b2 = b1; b2 < p->nblk; b2 += 2, ++g)
-                                load[g % sms] += (double)t * 0.5 * (std::min(2, p->nblk - b2) + (b2 != b1) + 1) +
-                                                 end + (sp[m] > 1 ? combine : 0.0);
-                        continue;
-                    }
-                    const int turn = group_turn((int)g, p->npairs, sms);
-                    for (int pr = 0; pr < p->npairs; ++pr, ++g)
-                        load[g % sms] +=
-                            (double)t * 0.5 * host_pair_units((pr + turn) % p->npairs, p->nblk) + end +
-                            (sp[m] > 1 ? combine : 0.0);
-                }
+                for (int k = 0; k < p->C; ++k)
+                    for (int b1 = 0; b1 < p->nblk; ++b1)
+                        for (int b2 = b1; b2 < p->nblk; b2 += 2, ++g) {
+                            const int w = p->nblk == 1 ? 2 : std::min(2, p->nblk - b2) + (b2 != b1) + 1;
+                            load[g % sms] += (double)t * 0.5 * w + 4.0 + (sp[m] > 1 ? 2.0 : 0.0);
+                        }
             }
         }
         const double score = *std::max_element(load.begin(), load.end());
@@ -1341,60 +1292,77 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
             best = sp;
         }
     }
-    out.sp = best;
+    cache.emplace_back(key, RangePlan{best, best_score});
+    if (cache.size() > 16) cache.erase(cache.begin());
+    return RangePlan{best, best_score};
+}
+
+// Work deal of one launch.  Round-robin: items go to the workers in turn, each
+// pass cut into `least` ranges (pass_ranges of the step's `total` modes), or,
+// single blocks, those of the launch's own modes where they are more.  Balanced
+// (a single-block mode alone): contiguous shares of the weighted k-tiles (see
+// next_piece), taken when cheaper in pass_ranges' cost model.  At N = 44, K =
+// 512 and 8192 frames per pass the round-robin deal leaves 104 CTAs with two
+// channels and 48 with one; the balanced deal gives each 1.7 channels.
+DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int64_t* S_pad, int total,
+                     const RangePlan& least) {
+    DealPlan out;
+    out.sp.resize(n);
+    if (lead->split > 0) {
+        // fixed by corr_set_tiles: round-robin, ranges per channel, at most one per k-tile
+        for (int m = 0; m < n; ++m) {
+            const int64_t tiles = std::max<int64_t>(1, S_pad[m] / plans[m]->KT);
+            out.sp[m] = (int)std::min<int64_t>(std::min(lead->split, plans[m]->max_split), tiles);
+        }
+        return out;
+    }
+    if (plans[0]->nblk > 1) {
+        out.sp.assign(least.sp.begin(), least.sp.begin() + n);
+        return out;
+    }
+    const RangePlan own = pass_ranges(plans, n, S_pad);
+    for (int m = 0; m < n; ++m) out.sp[m] = std::max(own.sp[m], least.sp[m]);
+    if (n > 1 || n < total) return out;
+    TcPlan* const p = plans[0];
+    for (auto& e : p->deal_cache)
+        if (e.first == S_pad[0]) return e.second;
+    const int sms = p->num_sms;
     // balanced deal: every CTA gets U/G units; an item then spans at most
     // (tiles - 1) w G / U + 2 CTAs, which must fit the partial slots, and a
-    // CTA holds at least 3 units (the heaviest k-tile), so it owns a k-tile of
+    // CTA holds at least 3 units (more than a k-tile's 2), so it owns a k-tile of
     // every item it overlaps and an item's CTAs are consecutive
-    int64_t units = 0, max_span = 0;
-    int cap_slots = 1 << 30;
-    for (int m = 0; m < n; ++m) {
-        const TcPlan* p = plans[m];
-        const int64_t tiles = S_pad[m] / p->KT;
-        for (int pr = 0; pr < p->npairs; ++pr) {
-            const int w = host_pair_units(pr, p->nblk);
-            units += item_units(tiles, w) * p->C;
-            if (tiles > 0) max_span = std::max<int64_t>(max_span, (tiles - 1) * w);
-        }
-        cap_slots = std::min(cap_slots, p->max_split);
-    }
     // (one mode only: with several, the round-robin deal spreads every mode's
     // items, whose ends differ in cost, evenly over the CTAs -- measured
     // faster on the four-mode batch)
     // (single antenna block only: with several, the round-robin deal hands one
     // channel's block pairs to neighbouring CTAs at once, which then share its
     // tiles through L2; contiguous shares would read them from HBM per pair)
-    if (n == 1 && plans[0]->nblk == 1 && units > 0 && cap_slots >= 3) {
+    const int64_t tiles = S_pad[0] / p->KT;
+    const int w = host_pair_units(0, 1);
+    const int64_t units = item_units(tiles, w) * p->C;
+    if (units > 0 && p->max_split >= 3) {
         int64_t G = sms;
-        if (max_span > 0)
-            G = std::min<int64_t>(G, std::max<int64_t>(1, (int64_t)(cap_slots - 2) * units / max_span));
+        const int64_t span = (tiles - 1) * w;
+        if (span > 0)
+            G = std::min<int64_t>(G, std::max<int64_t>(1, (int64_t)(p->max_split - 2) * units / span));
         G = std::min<int64_t>(G, std::max<int64_t>(1, units / 3));
         std::vector<double> bl(G, 0.0);
         int64_t ibase = 0;
-        for (int m = 0; m < n; ++m) {
-            const TcPlan* p = plans[m];
-            const int64_t tiles = S_pad[m] / p->KT;
-            if (tiles == 0) continue;
-            for (int pr = 0; pr < p->npairs; ++pr) {
-                const int w = host_pair_units(pr, p->nblk);
-                for (int k = 0; k < p->C; ++k, ibase += item_units(tiles, w)) {
-                    const int64_t t0 = ibase + kEndUnits;
-                    const int64_t first = t0 * G / units;
-                    const int64_t last = (t0 + (tiles - 1) * w) * G / units;
-                    for (int64_t j = 0; j < tiles; ++j) bl[(t0 + j * w) * G / units] += 0.5 * w;
-                    for (int64_t c = first; c <= last; ++c) bl[c] += 4.0 + (last > first ? 2.0 : 0.0);
-                }
-            }
+        for (int k = 0; k < p->C; ++k, ibase += item_units(tiles, w)) {
+            const int64_t t0 = ibase + kEndUnits;
+            const int64_t first = t0 * G / units;
+            const int64_t last = (t0 + span) * G / units;
+            for (int64_t j = 0; j < tiles; ++j) bl[(t0 + j * w) * G / units] += 0.5 * w;
+            for (int64_t c = first; c <= last; ++c) bl[c] += 4.0 + (last > first ? 2.0 : 0.0);
         }
-        const double score = *std::max_element(bl.begin(), bl.end());
-        if (score < best_score - 1e-9) {
+        if (*std::max_element(bl.begin(), bl.end()) < own.score - 1e-9) {
             out.balanced = true;
             out.grid = (int)G;
             out.units = units;
         }
     }
-    cache.emplace_back(key, out);
-    if (cache.size() > 16) cache.erase(cache.begin());
+    p->deal_cache.emplace_back(S_pad[0], out);
+    if (p->deal_cache.size() > 16) p->deal_cache.erase(p->deal_cache.begin());
     return out;
 }
 
@@ -1403,11 +1371,11 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
 namespace {
 
 // One kernel for plans that all have one antenna block, or all several.
-int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, cudaStream_t st,
-               std::string& err) {
+int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, int total,
+               const RangePlan& least, cudaStream_t st, std::string& err) {
     std::vector<int64_t> S(n);
     for (int m = 0; m < n; ++m) S[m] = runs[m]->S_pad;
-    const DealPlan deal = choose_deal(lead, plans, n, S.data(), runs[0]->stable);
+    const DealPlan deal = choose_deal(lead, plans, n, S.data(), total, least);
     const std::vector<int>& sp = deal.sp;
     const LaunchShape L = launch_shape(lead, plans, n);
     TcArgs a;
@@ -1460,11 +1428,11 @@ int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, cu
         d.unit_base = units;
         for (int pr = 0; pr < p->npairs; ++pr)
             units += item_units(d.tiles, host_pair_units(pr, p->nblk)) * p->C;
-        // single block: splits are combined inside the kernel, into acc;
-        // several blocks: every pass result lands in partial slot 0 (coalesced
-        // FP32 stores), which one reduction launch adds to acc
+        // single block: ranges are combined inside the kernel, into acc;
+        // several blocks: each range lands in its partial slot (coalesced FP32
+        // stores), and one reduction launch combines them
         runs[m]->direct = p->nblk == 1;
-        runs[m]->n_split = runs[m]->direct ? d.n_split : 1;
+        runs[m]->n_split = d.n_split;
     }
     a.total_items = base;
     // (largest dividend of the deal: units x CTAs plus a divisor)
@@ -1530,16 +1498,21 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
     // cta_group).  The lead's set goes first: a test hook on it fires there.
     TcPlan* set[kMaxTcModes];
     TcRun* srun[kMaxTcModes];
+    int64_t S[kMaxTcModes];
+    for (int m = 0; m < n; ++m) S[m] = runs[m].S_pad;
+    const RangePlan all = plans[0]->split > 0 ? RangePlan{} : pass_ranges(plans, n, S);
     const bool wide0 = plans[0]->nblk > 1;
     for (int pass = 0; pass < 2; ++pass) {
         int ns = 0;
+        RangePlan least;
         for (int m = 0; m < n; ++m)
             if ((plans[m]->nblk > 1) == (wide0 == (pass == 0))) {
+                if (!all.sp.empty()) least.sp.push_back(all.sp[m]);
                 set[ns] = plans[m];
                 srun[ns++] = &runs[m];
             }
         if (!ns) continue;
-        const int rc = launch_set(plans[0], set, ns, srun, st, err);
+        const int rc = launch_set(plans[0], set, ns, srun, n, least, st, err);
         if (rc != CORR_OK) return rc;
     }
     return CORR_OK;

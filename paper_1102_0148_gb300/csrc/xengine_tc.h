@@ -20,7 +20,6 @@ struct TcRun {
     const float* scale;       // [N][C] pre-cast scales (FP16 / FP8), else nullptr
     const float* split;       // [N] two-plane pre-scales sigma_i (FP32 mode), else nullptr
     int* status;              // device status word (bounded waits)
-    bool stable;              // ranges as a lone CTA's groups would take them (corr_set_stable)
     bool assign;              // acc holds zeros: the kernel may store instead of adding
     int n_split;              // out: partial slots the reduction adds (when !direct)
     bool direct;              // out: accumulated into acc in the kernel (single block)
