@@ -177,7 +177,11 @@ int corr_set_stable(corr_t h, int on);
 /* Correlate n samples per antenna (n a multiple of K, n >= 0) and add them
  * to the running integration.  `samples` holds n/K frames in the layout
  * above (n*N/2 bytes).  Host memory is staged through the handle's pinned
- * buffers; device memory is read in place.  With the fused F/X-engine on
+ * buffers; device memory is read in place.  Pushes of whole 128-frame blocks
+ * give the same spectra, to the bit, however many they are (an FP8 integration
+ * changes F-engine kernels at one of its frames, not of its pushes); a push of
+ * an odd number of frames may change the last bit of some FP32 spectra of the
+ * frames after it.  With the fused F/X-engine on
  * (corr_set_fused) device-memory pushes are recorded and queued as one
  * launch at the next corr_dump, corr_dump_async, corr_sync or call that
  * changes what they read (or when 262144 frames wait); their buffers must

@@ -98,7 +98,7 @@ struct corr_s {
     bool f_mma = false;              // which kind of kernel it was (fengine_mma_serves)
     cudaEvent_t f_span = nullptr;    // profiling: start of the open run of side launches
     bool stable = false;      // corr_set_stable
-    int64_t total = 0;        // frames of the integration with the push under way
+    int64_t pos = 0;          // frames of the integration before the next F-engine launch
     // coarse integer sample delays (corr_set_sample_delays)
     bool sdelay_on = false;
     int* sdelay = nullptr;          // [N] samples, device
@@ -397,13 +397,39 @@ FengineArgs fengine_args(corr_t h, const uint8_t* din, int64_t S, bool raw, int6
     fa.spec_type = h->spec_type;
     fa.scale = (h->spec_type == SPEC_F16 || h->spec_type == SPEC_F8) ? h->scale : nullptr;
     fa.split = split_table(h, raw);
-    fa.total = h->total;
+    fa.pos = h->pos;
     fa.stable = h->stable;
     fa.debug_out = nullptr;
     return fa;
 }
 
+// The first of S frames of the integration that belong to one kind of F-engine
+// kernel (an FP8 integration changes kinds at fp8_fft_frames).
+int64_t one_kind(corr_t h, const uint8_t* din, int64_t S) {
+    if (h->spec_type != SPEC_F8) return S;
+    const int64_t line = fp8_fft_frames(h->N);
+    if (h->pos >= line || h->pos + S <= line) return S;
+    FengineArgs fa = fengine_args(h, din, S, false, 0);
+    fa.pos = line;
+    return fengine_mma_serves(fa) ? line - h->pos : S;
+}
+
+// How many of S frames may go into one pass: one_kind's where the rest would
+// not start on a whole block of kSpecPad.
+int64_t one_pass(corr_t h, const uint8_t* din, int64_t S) {
+    const int64_t n = one_kind(h, din, S);
+    return n % kSpecPad ? n : S;
+}
+
 int fengine_pass(corr_t h, const uint8_t* din, int64_t S, bool raw, int64_t off) {
+    const int64_t n = one_kind(h, din, S);
+    if (n < S) {
+        int rc = fengine_pass(h, din, n, raw, off);
+        if (rc != CORR_OK) return rc;
+        // (in turn: what follows the second launch follows both)
+        CUDA_TRY(h, cudaStreamWaitEvent(h->f_stream[h->f_next], h->f_done[h->f_next ^ 1], 0));
+        return fengine_pass(h, din + n * ((int64_t)h->N * (h->K / 2)), S - n, raw, off + n);
+    }
     if (narrow(h) && !h->scales_ready) {
         int rc = estimate_scales(h, din, S);
         if (rc != CORR_OK) return rc;
@@ -429,6 +455,7 @@ int fengine_pass(corr_t h, const uint8_t* din, int64_t S, bool raw, int64_t off)
     h->f_pending[j] = true;
     h->f_next = j ^ 1;
     h->f_last = st;
+    h->pos += S;
     if (h->f_span) h->prof_launches[CORR_KERNEL_FENGINE] += 1;
     return CORR_OK;
 }
@@ -626,7 +653,7 @@ void free_stages(corr_t h) {
 // X-engine into `acc` whenever it fills up.
 int process_samples(corr_t h, const uint8_t* samples, int64_t n, bool raw, double2* acc) {
     const int64_t frames = n / h->K;
-    h->total = (raw ? 0 : h->n_spec) + frames;
+    h->pos = raw ? 0 : h->n_spec;
     const int64_t rec = (int64_t)h->N * (h->K / 2);
     const bool host = !is_device_ptr(samples);
     // (the fused F-engine reads 16 bytes per lane: 16-byte aligned input only)
@@ -666,6 +693,7 @@ int process_samples(corr_t h, const uint8_t* samples, int64_t n, bool raw, doubl
         const int64_t room = h->cap - h->fill;
         int64_t S = frames - f0 < room ? frames - f0 : room;
         if (host && S > h->stage_frames) S = h->stage_frames;
+        S = one_pass(h, host || h->sdelay_on ? nullptr : samples + f0 * rec, S);   // (buffers are aligned)
         const uint8_t* din = samples + f0 * rec;
         int b = 0;
         if (host) {
@@ -1534,13 +1562,17 @@ int batch_check(corr_batch_t b, const uint8_t* const* samples, const int64_t* n)
 // Queue every pass of every mode: per pass index, the F-engine of each mode
 // that has that pass, then one tensor-core launch over all of them.
 int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* n) {
-    int64_t frames[kMaxTcModes], passes = 0;
+    int64_t frames[kMaxTcModes], done[kMaxTcModes] = {};
     for (int m = 0; m < b->n; ++m) {
         frames[m] = n[m] / b->h[m]->K;
-        b->h[m]->total = b->h[m]->n_spec + frames[m];
-        passes = std::max(passes, (frames[m] + b->h[m]->cap - 1) / b->h[m]->cap);
+        b->h[m]->pos = b->h[m]->n_spec;
     }
-    for (int64_t pi = 0; pi < passes; ++pi) {
+    auto left = [&] {
+        for (int m = 0; m < b->n; ++m)
+            if (done[m] < frames[m]) return true;
+        return false;
+    };
+    while (left()) {
         TcPlan* plans[kMaxTcModes];
         TcRun runs[kMaxTcModes];
         int idx[kMaxTcModes];
@@ -1548,10 +1580,12 @@ int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* 
         FengineArgs fas[kMaxTcModes];
         for (int m = 0; m < b->n; ++m) {
             corr_t h = b->h[m];
-            const int64_t f0 = pi * h->cap;
+            const int64_t f0 = done[m];
             if (f0 >= frames[m]) continue;
-            const int64_t S = std::min(h->cap, frames[m] - f0);
+            int64_t S = std::min(h->cap, frames[m] - f0);
             const int64_t rec = (int64_t)h->N * (h->K / 2);
+            if (!b->one_f) S = one_pass(h, samples[m] + f0 * rec, S);
+            done[m] += S;
             if (b->one_f) {
                 if (narrow(h) && !h->scales_ready) {
                     int rc = estimate_scales(h, samples[m] + f0 * rec, S);

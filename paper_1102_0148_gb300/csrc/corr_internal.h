@@ -100,7 +100,7 @@ struct FengineArgs {
     // Set by launch_fengine: the K = 512 grid runs antenna fastest
     // (blockIdx.x = antenna) unless its frame blocks exceed gridDim.y's limit.
     int ant_x;
-    int64_t total;           // frames of the integration with this push (0: S)
+    int64_t pos;             // frames of the integration before these
     int stable;              // FP32 and pair outputs from the FP32 kernels (corr_set_stable)
 };
 
@@ -108,6 +108,9 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st);
 // The kernels with a tensor-core first stage (fengine_mma.cu), and whether
 // they serve these arguments (K, output type, input alignment).
 bool fengine_mma_serves(const FengineArgs& a);
+// Frames of an FP8 integration, from its first, that keep the FP32 FFTs
+// whatever the pushes: a whole number of kSpecPad.
+int64_t fp8_fft_frames(int N);
 cudaError_t launch_fengine_mma(const FengineArgs& a, cudaStream_t st);
 // The F-engines of n modes (1 <= n <= 4, one workspace element type, no
 // debug output) as one launch: each mode's frames as its own kernel would

@@ -972,16 +972,24 @@ cudaError_t launch_shape(const FengineArgs& a, cudaStream_t st) {
 
 }  // namespace
 
+// One E4M3 rounding that falls the other way moves a visibility by up to ~0.45
+// of a sample's power, 0.45 / (T sqrt(2 / N + 1 / T)) of the rms visibility of T
+// spectra: in short integrations the two kinds of kernel, equally accurate,
+// differ by 1e-3 of it (N = 44, T = 2048) to 4e-3 (N = 11, T = 120).  So an FP8
+// integration starts on the FP32 FFTs, and its frames go over to the others
+// where 2 T^2 / N + T = 420000 (N = 44: 3072 frames), from where it stays below
+// 7e-4.  The line is one of the integration's frames, not of the pushes: the
+// same samples round alike however they are pushed.  FP16's roundings are 64
+// times finer.
+int64_t fp8_fft_frames(int N) {
+    int64_t T = kSpecPad;
+    while (2.0 * (double)T * T / N + T < 420000.0) T += kSpecPad;
+    return T;
+}
+
 bool fengine_mma_serves(const FengineArgs& a) {
     if (a.K < 16 || a.K > 2048) return false;
-    // FP8 in short integrations keeps the FP32 FFTs' roundings: one E4M3
-    // rounding that falls the other way moves a visibility by up to ~0.45 of a
-    // sample's power, 0.45 / (T sqrt(2 / N + 1 / T)) of the rms visibility of T
-    // spectra.  From here on that is below 7e-4 (N = 44: T >= 3018); 1e-3 was
-    // seen at N = 44, T = 2048 and 4e-3 at N = 11, T = 120.  T: what this push
-    // brings the integration to.  FP16's roundings are 64 times finer.
-    const double T = (double)std::max(a.total, a.S);
-    if (a.spec_type == SPEC_F8 && !a.debug_out && 2.0 * T * T / a.N + T < 420000.0) return false;
+    if (a.spec_type == SPEC_F8 && !a.debug_out && a.pos < fp8_fft_frames(a.N)) return false;
     if (a.stable && (a.spec_type == SPEC_F32 || a.spec_type == SPEC_F16X2)) return false;
     // bytes of the widest load: one pair of n1, at least a cp.async for K >= 512
     const uintptr_t align = a.K >= 512 ? 16 : (a.K <= 32 ? 1 : a.K / 32);
