@@ -46,6 +46,31 @@ __device__ __forceinline__ void store_spec(void* spec, int t, int64_t off, float
     }
 }
 
+// Four adjacent frames (off a multiple of 4).
+__device__ __forceinline__ void store_spec4(void* spec, int t, int64_t off, float4 v, int64_t plane_stride,
+                                            float sigma) {
+    auto pair = [](float a, float b) {
+        const __half2 h = __floats2half2_rn(a, b);
+        return *reinterpret_cast<const uint32_t*>(&h);
+    };
+    if (t == SPEC_F32) {
+        *reinterpret_cast<float4*>(static_cast<float*>(spec) + off) = v;
+    } else if (t == SPEC_F16X2) {
+        v = make_float4(v.x * sigma, v.y * sigma, v.z * sigma, v.w * sigma);
+        const __half2 h0 = __floats2half2_rn(v.x, v.y), h1 = __floats2half2_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(static_cast<__half*>(spec) + off) = make_uint2(pair(v.x, v.y), pair(v.z, v.w));
+        *reinterpret_cast<uint2*>(static_cast<__half*>(spec) + off + plane_stride) =
+            make_uint2(pair(v.x - __low2float(h0), v.y - __high2float(h0)),
+                       pair(v.z - __low2float(h1), v.w - __high2float(h1)));
+    } else if (t == SPEC_F16) {
+        *reinterpret_cast<uint2*>(static_cast<__half*>(spec) + off) = make_uint2(pair(v.x, v.y), pair(v.z, v.w));
+    } else {
+        const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v.x, v.y), __NV_SATFINITE, __NV_E4M3);
+        const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(v.z, v.w), __NV_SATFINITE, __NV_E4M3);
+        *reinterpret_cast<uint32_t*>(static_cast<__nv_fp8_storage_t*>(spec) + off) = lo | hi << 16;
+    }
+}
+
 // Real transform of one frame, for k = tid, tid + kThreads, ...: the
 // complex transform Z (natural order, length L) is in `Z`.
 __device__ __forceinline__ float2 real_split(const float2* Z, int k, int L, const float2* tw) {
@@ -58,10 +83,58 @@ __device__ __forceinline__ float2 real_split(const float2* Z, int k, int L, cons
     return make_float2(E.x + t.x, E.y + t.y);
 }
 
+// One frame of antenna i by `threads` threads (tid): a radix-2 Stockham FFT in
+// shared memory (x, y: L values each), the real split and the correction, then
+// out(k, X).  `sync` is a barrier of those threads; stage_tw(Ns, j) is W_{2Ns}^j,
+// split_tw[k] W_K^k.
+template <class Sync, class Tw, class Out>
+__device__ __forceinline__ void fgeneric_frame(const FengineArgs& a, int i, const uint8_t* src, bool valid,
+                                               float2* x, float2* y, int tid, int threads, Sync sync,
+                                               Tw stage_tw, const float2* split_tw, Out out) {
+    const int L = a.K >> 1;
+    for (int m = tid; m < L; m += threads) {
+        float2 z = make_float2(0.f, 0.f);
+        if (valid) {
+            const unsigned b = src[m];
+            z = make_float2(nib(b & 15u), nib(b >> 4));
+        }
+        x[m] = z;
+    }
+    sync();
+    for (int Ns = 1; Ns < L; Ns <<= 1) {
+        for (int j = tid; j < (L >> 1); j += threads) {
+            const int kk = j & (Ns - 1);
+            const float2 v0 = x[j];
+            const float2 v1 = cmul(x[j + (L >> 1)], stage_tw(Ns, kk));
+            const int d = ((j - kk) << 1) + kk;
+            y[d] = make_float2(v0.x + v1.x, v0.y + v1.y);
+            y[d + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
+        }
+        sync();
+        float2* t = x;
+        x = y;
+        y = t;
+    }
+    for (int k = tid; k < L; k += threads) {
+        float2 X = real_split(x, k, L, split_tw);
+        if (a.corr) X = cmul(a.corr[(int64_t)i * L + k], X);
+        out(k, X);
+    }
+    sync();
+}
+
+__device__ __forceinline__ float2 prescaled(const FengineArgs& a, int i, int k, float2 X) {
+    if (a.scale) {
+        const float sc = a.scale[(int64_t)i * (a.K >> 1) + k];
+        X.x *= sc;
+        X.y *= sc;
+    }
+    return X;
+}
+
 // Generic F-engine for any power-of-two K: one CTA transforms FT frames of one
-// antenna, one frame at a time, with a radix-2 Stockham FFT in shared memory;
-// the FT results of each channel are staged and written as one contiguous run
-// of the workspace row (k, r).
+// antenna, one frame at a time; the FT results of each channel are staged and
+// written as one contiguous run of the workspace row (k, r).
 // The body: FT frames from s0 of antenna i by kThreads threads (tid), `smem`
 // 16 L + (DEBUG ? 0 : 8 C FT) bytes, `sync` a barrier of those threads.
 template <bool DEBUG, class Sync>
@@ -77,50 +150,17 @@ __device__ __forceinline__ void fgeneric_block(const FengineArgs& a, int FT, int
     for (int f = 0; f < FT; ++f) {
         const int64_t s = s0 + f;
         if (s >= s_end) break;                              // uniform in the CTA
-        const bool valid = s < a.S;
-        const uint8_t* src = a.in + (s * a.N + i) * (int64_t)L;
-        for (int m = tid; m < L; m += kThreads) {
-            float2 z = make_float2(0.f, 0.f);
-            if (valid) {
-                const unsigned b = src[m];
-                z = make_float2(nib(b & 15u), nib(b >> 4));
-            }
-            bufA[m] = z;
-        }
-        sync();
-        float2* x = bufA;
-        float2* y = bufB;
-        for (int Ns = 1; Ns < L; Ns <<= 1) {
-            const int tstep = a.K / (2 * Ns);              // W_{2Ns}^j = W_K^{j K/(2Ns)}
-            for (int j = tid; j < (L >> 1); j += kThreads) {
-                const int kk = j & (Ns - 1);
-                const float2 v0 = x[j];
-                const float2 v1 = cmul(x[j + (L >> 1)], a.twiddle[kk * tstep]);
-                const int d = ((j - kk) << 1) + kk;
-                y[d] = make_float2(v0.x + v1.x, v0.y + v1.y);
-                y[d + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
-            }
-            sync();
-            float2* t = x;
-            x = y;
-            y = t;
-        }
-        for (int k = tid; k < C; k += kThreads) {
-            float2 X = real_split(x, k, L, a.twiddle);
-            if (a.corr) X = cmul(a.corr[(int64_t)i * C + k], X);
-            if (DEBUG) {
-                a.debug_out[((int64_t)i * a.S + s) * C + k] = X;
-            } else {
-                if (a.scale) {
-                    const float sc = a.scale[(int64_t)i * C + k];
-                    X.x *= sc;
-                    X.y *= sc;
+        fgeneric_frame(
+            a, i, a.in + (s * a.N + i) * (int64_t)L, s < a.S, bufA, bufB, tid, kThreads, sync,
+            [&](int Ns, int j) { return a.twiddle[j * (a.K / (2 * Ns))]; }, a.twiddle, [&](int k, float2 X) {
+                if (DEBUG) {
+                    a.debug_out[((int64_t)i * a.S + s) * C + k] = X;
+                } else {
+                    X = prescaled(a, i, k, X);
+                    stg[k * FT + f] = X.x;
+                    stg[(C + k) * FT + f] = X.y;
                 }
-                stg[k * FT + f] = X.x;
-                stg[(C + k) * FT + f] = X.y;
-            }
-        }
-        sync();
+            });
     }
     if (!DEBUG) {
         const float sigma = a.spec_type == SPEC_F16X2 ? __ldg(a.split + i) : 1.0f;
@@ -143,6 +183,68 @@ __global__ void __launch_bounds__(kThreads) fengine_generic(FengineArgs a, int F
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fgeneric_block<DEBUG>(a, FT, blockIdx.y, (int64_t)blockIdx.x * FT, smem_raw, threadIdx.x,
                           []() { __syncthreads(); });
+}
+
+// K <= 256, where a frame has work for a warp at most: the same arithmetic with
+// 8 to 32 lanes per frame and no CTA barriers between stages, 32 frames of an
+// antenna per CTA.  The first frames of FP8 integrations, stable FP32 outputs
+// and unaligned input run here, to the bit as in the body above, whose 256
+// threads had a barrier for every stage of each frame.  Twiddles come from
+// shared memory, each stage's adjacent; staging rows are a float longer than 32
+// frames (the writes of a channel's frames hit one bank otherwise).  Bound by
+// issue.  64 antennas FP8, F-engine: K = 128, 2048 frames 381 -> 71 us; K = 256,
+// 16384 frames (3712 of them here) 1089 -> 349.
+constexpr int kSmallFrames = 32;
+
+__host__ __device__ __forceinline__ int small_lanes(int K) { return K <= 32 ? 8 : (K == 64 ? 16 : 32); }
+size_t small_smem(int K, bool debug) {
+    return (size_t)K * sizeof(float2) + (size_t)(kThreads / small_lanes(K)) * K * sizeof(float2) +
+           (debug ? 0 : (size_t)K * (kSmallFrames + 1) * sizeof(float));
+}
+
+template <bool DEBUG>
+__global__ void __launch_bounds__(kThreads) fengine_small(FengineArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = a.K >> 1, G = small_lanes(a.K);
+    const int i = blockIdx.y, grp = threadIdx.x / G, t = threadIdx.x % G;
+    const int64_t s0 = (int64_t)blockIdx.x * kSmallFrames;
+    float2* tw = reinterpret_cast<float2*>(smem_raw);      // W_K^k, k < L; W_{2Ns}^j at L + Ns + j
+    float2* buf = tw + a.K + grp * a.K;
+    float* stg = reinterpret_cast<float*>(tw + a.K + (kThreads / G) * a.K);
+    for (int e = threadIdx.x; e < a.K; e += kThreads) {
+        const int Ns = e <= L ? 1 : 1 << (31 - __clz(e - L));
+        tw[e] = a.twiddle[e < L ? e : (e == L ? 0 : (e - L - Ns) * (a.K / (2 * Ns)))];
+    }
+    __syncthreads();
+    const int64_t s_end = DEBUG ? a.S : a.S_pad;
+    for (int f = grp; f < kSmallFrames; f += kThreads / G) {
+        const int64_t s = s0 + f;
+        fgeneric_frame(
+            a, i, a.in + (s * a.N + i) * (int64_t)L, s < a.S, buf, buf + L, t, G, []() { __syncwarp(); },
+            [&](int Ns, int j) { return tw[L + Ns + j]; }, tw, [&](int k, float2 X) {
+                if (s >= s_end) return;
+                if (DEBUG) {
+                    a.debug_out[((int64_t)i * a.S + s) * L + k] = X;
+                } else {
+                    X = prescaled(a, i, k, X);
+                    stg[k * (kSmallFrames + 1) + f] = X.x;
+                    stg[(L + k) * (kSmallFrames + 1) + f] = X.y;
+                }
+            });
+    }
+    __syncthreads();
+    if (DEBUG) return;
+    // four frames of a row per thread and store (S_pad is a multiple of 4)
+    const float sigma = a.spec_type == SPEC_F16X2 ? __ldg(a.split + i) : 1.0f;
+    for (int e = threadIdx.x; e < a.K * (kSmallFrames / 4); e += kThreads) {
+        const int row = e >> 3, f = (e & 7) * 4;
+        if (s0 + f >= a.S_pad) continue;
+        const float* v = stg + row * (kSmallFrames + 1) + f;
+        const int plane = row >= L;
+        const int64_t off = spec_off(row - plane * L, spec_row(plane, i, a.N), a.s_base + s0 + f, a.N, L,
+                                     spec_tile_shift(a.spec_type));
+        store_spec4(a.spec, a.spec_type, off, make_float4(v[0], v[1], v[2], v[3]), a.plane_stride, sigma);
+    }
 }
 
 // K = 512 kernel: one 32-frame block of one antenna per CTA (the body is
@@ -788,10 +890,21 @@ cudaError_t launch_fengine(const FengineArgs& a, cudaStream_t st) {
             default: return go(fengine_rad16<8, SPEC_F16X2>);
         }
     }
-    int FT = 8192 / C;
-    FT = FT < 1 ? 1 : (FT > 32 ? 32 : FT);
     const int64_t frames = dbg ? a.S : a.S_pad;
     if (frames <= 0) return cudaSuccess;
+    if (a.K <= 256) {
+        const size_t smem = small_smem(a.K, dbg);
+        const dim3 grid((unsigned)((frames + kSmallFrames - 1) / kSmallFrames), (unsigned)a.N);
+        auto go = [&](auto kern) -> cudaError_t {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            kern<<<grid, kThreads, smem, st>>>(a);
+            return cudaGetLastError();
+        };
+        return dbg ? go(fengine_small<true>) : go(fengine_small<false>);
+    }
+    int FT = 8192 / C;
+    FT = FT < 1 ? 1 : (FT > 32 ? 32 : FT);
     const size_t smem = (size_t)16 * L + (dbg ? 0 : (size_t)8 * C * FT);
     dim3 grid((unsigned)((frames + FT - 1) / FT), (unsigned)a.N);
     cudaError_t e;
