@@ -166,13 +166,14 @@ int corr_get_scales(corr_t h, float* scales);
  * batches (corr_batch_*) reject handles with delays set (CORR_EINVAL). */
 int corr_set_sample_delays(corr_t h, const int32_t* delays);
 
-/* on: later pushes and passes of an FP32 handle round as the FP32 kernels
- * always have (FFTs in FP32 throughout), so
- * FP64 visibilities stay the same to the bit from one version to the next, as
- * a loss and its finite differences want; off (the default): the fastest
- * kernels, equally accurate.  The autograd binding turns it on for its
- * forward pass. */
+/* on: later pushes of an FP32 handle (CORR_FP32 or CORR_FP32_SIMT) take FFTs
+ * that round in FP32 throughout, one frame apart from the other, at every K;
+ * off (the default): the fastest kernels, equally accurate, which for K <= 256
+ * and K = 2048 have a tensor-core first stage.  The autograd binding turns it
+ * on for its forward pass, whose loss is often differenced, and puts the
+ * handle's own setting back.  corr_get_stable: *on = 0 or 1. */
 int corr_set_stable(corr_t h, int on);
+int corr_get_stable(corr_t h, int* on);
 
 /* Correlate n samples per antenna (n a multiple of K, n >= 0) and add them
  * to the running integration.  `samples` holds n/K frames in the layout

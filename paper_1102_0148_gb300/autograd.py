@@ -37,12 +37,13 @@ class Visibilities(torch.autograd.Function):
         corr.corr_set_corrections(c.h, g, t)
         n = samples.numel() * 2 // c.N
         V = torch.empty((c.P, c.C), dtype=torch.complex128, device=samples.device)
+        stable = corr.corr_get_stable(c.h)
         corr.corr_set_stable(c.h, True)
         try:
             corr.corr_push(c.h, samples, n)
             corr.corr_dump(c.h, V, fp64=True)
         finally:
-            corr.corr_set_stable(c.h, False)
+            corr.corr_set_stable(c.h, stable)
         ctx.save_for_backward(g, t, samples)
         ctx.c = c
         ctx.n = n

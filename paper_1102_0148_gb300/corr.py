@@ -60,6 +60,7 @@ _SIGS = {
     "corr_set_scales": (_int, [_vp, _vp]),
     "corr_set_sample_delays": (_int, [_vp, _vp]),
     "corr_set_stable": (_int, [_vp, _int]),
+    "corr_get_stable": (_int, [_vp, ctypes.POINTER(_int)]),
     "corr_batch_create": (_int, [ctypes.POINTER(_vp), _int, ctypes.POINTER(_int), ctypes.POINTER(_int), _int]),
     "corr_batch_set_chunk": (_int, [_vp, _i64]),
     "corr_batch_set_tiles": (_int, [_vp, _int, _int, _int, _int]),
@@ -211,8 +212,14 @@ def corr_set_sample_delays(h, delays):
 
 
 def corr_set_stable(h, on):
-    """Round as the FP32 kernels always have (on), or take the fastest ones."""
+    """FFTs that round in FP32 throughout (on), or the fastest ones."""
     return _check(_lib.corr_set_stable(h, 1 if on else 0), h)
+
+
+def corr_get_stable(h):
+    on = _int()
+    _check(_lib.corr_get_stable(h, ctypes.byref(on)), h)
+    return bool(on.value)
 
 
 def corr_dump_async(h, vis, fp64=False):

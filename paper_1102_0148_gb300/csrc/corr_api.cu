@@ -1157,6 +1157,12 @@ int corr_set_stable(corr_t h, int on) {
     return CORR_OK;
 }
 
+int corr_get_stable(corr_t h, int* on) {
+    if (!h || !on) return CORR_EINVAL;
+    *on = h->stable ? 1 : 0;
+    return CORR_OK;
+}
+
 int corr_set_sample_delays(corr_t h, const int32_t* delays) {
     if (!h) return CORR_EINVAL;
     std::vector<int> d(h->N, 0);
