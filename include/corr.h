@@ -314,15 +314,19 @@ int corr_debug_spectra(corr_t h, const uint8_t* samples, int64_t n, float* spect
 
 /* ------------------------------------------------------------------------
  * Batches: several correlators ("modes", e.g. sub-arrays with different N
- * and K) whose X-engine work runs as ONE persistent tensor-core launch per
- * pass (no counterpart in the paper, whose correlator serves one mode).
+ * and K) whose X-engine work shares persistent tensor-core launches (no
+ * counterpart in the paper, whose correlator serves one mode): per pass one
+ * for the modes of up to 64 antennas and one for the larger ones, whose work
+ * goes to pairs of CTAs.
  * All modes share the X-engine precision (CORR_FP32, CORR_FP16 or
  * CORR_FP8E4M3) and one non-blocking stream owned by the batch; each mode
  * keeps its own workspace and FP64 accumulators.  Per pass index the
  * F-engine of every mode that has that pass is queued (the modes' F-engines
- * run side by side on their handles' side streams), then one launch covers
- * all of their X-engine work.  With each mode's chunk at least its
- * push size (corr_batch_set_chunk), a push is exactly one X-engine launch.
+ * run side by side on their handles' side streams), then these launches cover
+ * all of their X-engine work.  With each mode's chunk at least its push size
+ * (corr_batch_set_chunk) a push is one pass; an FP8 mode takes a second one
+ * where its F-engine kernels change within a 128-frame block (corr_push).
+ * corr_profile_read of mode 0 counts the launches.
  *
  * corr_batch_create  n_modes in [1, 4]; N[m], K[m] as corr_create.
  * corr_batch_push    samples[m]: device buffer of n[m] samples per antenna of
@@ -345,12 +349,13 @@ int corr_debug_spectra(corr_t h, const uint8_t* samples, int64_t n, float* spect
  * corr_batch_set_one_launch  on = 1: each pass runs the F-engines of all its
  *                    modes as one launch (a persistent kernel of 768-thread
  *                    CTAs, three 256-thread sub-blocks for K = 512, 1024 and
- *                    other K, 512 threads for K = 2048 / 4096), so a step is
- *                    one F-engine and one X-engine launch; on = 0 (the
- *                    default): one launch per mode, side by side.  On a
- *                    GB300 the single launch is ~15% slower on the batching
- *                    workload (its union kernel is held to 80 registers and
- *                    spills); results are the same.  Switching discards a
+ *                    other K, 512 threads for K = 2048 / 4096); on = 0 (the
+ *                    default): one launch per mode, side by side.  The single
+ *                    launch takes the FP32 FFTs of every K (spectra as accurate,
+ *                    but FP16 / FP8 values may round otherwise), and its union
+ *                    kernel is held to 80 registers and spills: a step of the
+ *                    batching workload takes 2.85 ms in FP16 against 2.08 ms,
+ *                    4.21 in FP32 mode against 3.61.  Switching discards a
  *                    recorded graph.
  * Errors: as the single-mode calls; corr_batch_last_error(b) has the message
  * (corr_last_error(NULL) for corr_batch_create). */

@@ -418,8 +418,9 @@ class Correlator:
 
 
 class CorrelatorBatch:
-    """Several correlators of uneven N and K whose X-engine work shares one
-    persistent tensor-core launch per pass (optionally replayed as a CUDA
+    """Several correlators of uneven N and K whose X-engine work shares
+    persistent tensor-core launches, per pass one for the modes of up to 64
+    antennas and one for the larger ones (optionally replayed as a CUDA
     graph)."""
 
     def __init__(self, modes, dtype=CORR_FP32, chunk=None, window=0, stages=0, split=0,

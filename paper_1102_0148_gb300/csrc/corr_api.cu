@@ -297,14 +297,14 @@ void prof_begin(corr_t h) {
     if (h->ev_open) cudaEventRecord(h->ev_open, h->stream);
 }
 
-void prof_end(corr_t h, int cls) {
+void prof_end(corr_t h, int cls, int launches = 1) {
     if (!h->prof_on || !h->ev_open) return;
     cudaEvent_t e = prof_event(h);
     if (!e) return;
     cudaEventRecord(e, h->stream);
     h->ev_pending[cls].emplace_back(h->ev_open, e);
     h->ev_open = nullptr;
-    h->prof_launches[cls] += 1;
+    h->prof_launches[cls] += launches;
 }
 
 // Make the handle's stream wait for the F-engine launches on the side
@@ -1566,7 +1566,7 @@ int batch_check(corr_batch_t b, const uint8_t* const* samples, const int64_t* n)
 }
 
 // Queue every pass of every mode: per pass index, the F-engine of each mode
-// that has that pass, then one tensor-core launch over all of them.
+// that has that pass, then the tensor-core launches over all of them.
 int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* n) {
     int64_t frames[kMaxTcModes], done[kMaxTcModes] = {};
     for (int m = 0; m < b->n; ++m) {
@@ -1632,15 +1632,16 @@ int batch_enqueue(corr_batch_t b, const uint8_t* const* samples, const int64_t* 
                 if (rc != CORR_OK) return batch_from_handle(b, idx[a], rc);
             }
         }
-        // one tensor-core launch over all of them (it overwrites their partials)
+        // the tensor-core launches over all of them (they overwrite their partials)
         for (int a = 0; a < na; ++a) {
             int src = settle_partial(b->h[idx[a]]);
             if (src != CORR_OK) return batch_from_handle(b, idx[a], src);
         }
         prof_begin(h0);
-        int rc = tc_launch(plans, na, runs, b->stream, b->err);
+        int launches = 0;
+        int rc = tc_launch(plans, na, runs, b->stream, b->err, &launches);
         if (rc != CORR_OK) return rc;
-        prof_end(h0, CORR_KERNEL_XENGINE);
+        prof_end(h0, CORR_KERNEL_XENGINE, launches);
         for (int a = 0; a < na; ++a) {
             rc = finish_tc_run(b->h[idx[a]], runs[a], b->h[idx[a]]->acc);
             if (rc != CORR_OK) return batch_from_handle(b, idx[a], rc);

@@ -113,8 +113,8 @@ bool fengine_mma_serves(const FengineArgs& a);
 int64_t fp8_fft_frames(int N);
 cudaError_t launch_fengine_mma(const FengineArgs& a, cudaStream_t st);
 // The F-engines of n modes (1 <= n <= 4, one workspace element type, no
-// debug output) as one launch: each mode's frames as its own kernel would
-// transform them.
+// debug output) as one launch, on the FP32 FFTs of every K (never the kernels
+// with a tensor-core first stage).
 cudaError_t launch_fengine_multi(const FengineArgs* modes, int n, cudaStream_t st);
 
 // Coarse integer delays on the packed stream: out = in delayed by delays[i]

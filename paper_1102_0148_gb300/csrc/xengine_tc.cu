@@ -1478,7 +1478,8 @@ int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, in
 
 }  // namespace
 
-int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err) {
+int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err, int* launches) {
+    if (launches) *launches = 0;
     if (n < 1 || n > kMaxTcModes) {
         err = "between 1 and 4 modes per tensor-core launch";
         return CORR_EINVAL;
@@ -1514,6 +1515,7 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
         if (!ns) continue;
         const int rc = launch_set(plans[0], set, ns, srun, n, least, st, err);
         if (rc != CORR_OK) return rc;
+        if (launches) ++*launches;
     }
     return CORR_OK;
 }

@@ -38,7 +38,9 @@ int tc_set_tiles(TcPlan* p, int window, int stages, int split, int atoms, std::s
 // are those of plans[0].
 // Modes whose run reports direct = false need the reduction of their
 // n_split partial blocks into acc.
-int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err);
+// *launches (when not nullptr): how many launches that took.
+int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::string& err,
+              int* launches = nullptr);
 // Test hook: the next launch's CTA 0 skips the copies of its first stage, so
 // its MMA warp's bounded wait expires after wait_limit_s.
 int tc_test_withhold(TcPlan* p, double wait_limit_s, std::string& err);
