@@ -267,7 +267,11 @@ int corr_load_state(corr_t h, const void* buf);
  * the k-th allocation counted since the variable last changed value fails
  * as if the device were out of memory.  The call that made it returns
  * CORR_ENOMEM with nothing half-allocated and the handle still usable.
- * (corr_correlate_noalloc allocates nothing and is not affected.) */
+ * (corr_correlate_noalloc allocates nothing and is not affected.)
+ * While CORR_TEST_NO_TENSOR_MAPS is set, the driver's tensor-map encoder is
+ * looked up as if it were missing (a process that has found it keeps it):
+ * CORR_FP32_SIMT handles and corr_correlate_noalloc work without it, the other
+ * types report CORR_ECUDA at corr_create. */
 
 /* Test hook for the failure path (no counterpart in the paper).  kind 1: in
  * the next tensor-core X-engine launch, the first work item of CTA 0 never

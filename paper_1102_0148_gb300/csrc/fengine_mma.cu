@@ -994,9 +994,10 @@ bool fengine_mma_serves(const FengineArgs& a) {
     // bytes of the widest load: one pair of n1, at least a cp.async for K >= 512
     const uintptr_t align = a.K >= 512 ? 16 : (a.K <= 32 ? 1 : a.K / 32);
     if (reinterpret_cast<uintptr_t>(a.in) % align) return false;
-    if (a.K == 512 || a.K == 1024)
-        return !a.debug_out && (a.spec_type == SPEC_F16 || a.spec_type == SPEC_F8);
-    return true;
+    if ((a.K == 512 || a.K == 1024) && (a.debug_out || (a.spec_type != SPEC_F16 && a.spec_type != SPEC_F8)))
+        return false;
+    // (without tensor maps only FP32 outputs exist: the other types' handles need them)
+    return a.debug_out || tc::get_encoder();
 }
 
 cudaError_t launch_fengine_mma(const FengineArgs& a, cudaStream_t st) {

@@ -10,6 +10,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <cstdlib>
 
 namespace gbcorr {
 namespace tc {
@@ -249,6 +250,7 @@ inline PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
     static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> known{nullptr};
     PFN_cuTensorMapEncodeTiled_v12000 fn = known.load(std::memory_order_acquire);
     if (fn) return fn;
+    if (std::getenv("CORR_TEST_NO_TENSOR_MAPS")) return nullptr;      // test hook
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
