@@ -32,9 +32,12 @@
 // frame and n2: two nibbles of equal position in two words, one PRMT and one
 // LOP3 away from the packed bytes.  A nibble u = v + 8 becomes the FP16
 // subnormal u 2^-24 (or 16 u 2^-24 from a high nibble: odd n2), which the MMA
-// takes as it is; the twiddles carry 2^24 (2^20 for odd n2), the rows of the
-// matrix sum to zero exactly, and the accumulator of row k1 = 0 starts at
-// minus the offset.
+// takes as it is; the twiddles carry 2^24 (2^20 for odd n2).  The offset of 8
+// is the same for every n1 and n2, so it drops out of every row but k1 = 0 (the
+// others sum to zero exactly) and, in row k1 = 0, out of every channel
+// but X[0]: that row's twiddles are 1 and its first butterflies add and
+// subtract integers, so its differences lose the offset exactly before any
+// other factor.  X[0] has it subtracted after stage 2.
 //
 // k1 = 0 and N1/2 share the row pair g = 0 of m-tile 0 as real sequences.  Its
 // lanes swap them so that one complex transform holds the k1 = 0 sequences of
@@ -233,13 +236,6 @@ __device__ __forceinline__ void stmatrix2(uint32_t addr, uint32_t r0, uint32_t r
     asm volatile("stmatrix.sync.aligned.m8n8.x2.shared.b16 [%0], {%1,%2};" ::"r"(addr), "r"(r0),
                  "r"(r1)
                  : "memory");
-}
-
-// One lane of the (converged) warp, the same one each time.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{.reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;}" : "=r"(p));
-    return p != 0;
 }
 
 // half2 (lo half = a)
@@ -850,7 +846,7 @@ fengine_mma(const __grid_constant__ FengineArgs a, const __grid_constant__ OutMa
             // the staged boxes go out by TMA, one lane of each warp issuing
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
-            if (elect_one()) {
+            if (tc::elect_one()) {
                 constexpr int tsh = OUT == SPEC_F8 ? 7 : 5;
                 const int64_t s = a.s_base + (int64_t)fb * kMmaFrames;
                 const int tile = (int)(s >> tsh), x = (int)(s & ((1 << tsh) - 1));

@@ -162,7 +162,7 @@ __device__ __forceinline__ uint64_t op_desc(uint32_t lo) {
     return (uint64_t)hi << 32 | lo;
 }
 
-// One lane of a converged warp.
+// One lane of a converged warp, the same one each time.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile(

@@ -100,7 +100,6 @@ struct TcArgs {
     int kt_shift;             // log2(KT): the single-lane roles avoid 64-bit division
     int atoms;                // k-tiles of KT spectra per pipeline stage
     int row_bytes;            // bytes of one tile row: 64 (FP16 modes) or 128 (FP8)
-    int wide;                 // modes of several antenna blocks: atoms hold A and B slots
     int gs_floats;            // epilogue G buffer (largest 2nb x (2nb + 1) of the modes; FP32 mode + 2 kRows)
     int slot_rows;            // rows of one operand tile slot in shared memory (<= 128)
     int* status;
@@ -1387,7 +1386,6 @@ int launch_set(TcPlan* lead, TcPlan* const* plans, int n, TcRun* const* runs, in
     a.row_bytes = plans[0]->row_bytes;
     a.W = L.W;
     a.atoms = L.atoms;
-    a.wide = L.wide;
     a.gs_floats = L.gs_floats;
     a.slot_rows = L.slot_rows;
     a.status = runs[0]->status;
