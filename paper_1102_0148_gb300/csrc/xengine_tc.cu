@@ -1319,12 +1319,16 @@ DealPlan choose_deal(const TcPlan* lead, TcPlan* const* plans, int n, const int6
         out.sp.assign(least.sp.begin(), least.sp.begin() + n);
         return out;
     }
-    const RangePlan own = pass_ranges(plans, n, S_pad);
-    for (int m = 0; m < n; ++m) out.sp[m] = std::max(own.sp[m], least.sp[m]);
-    if (n > 1 || n < total) return out;
     TcPlan* const p = plans[0];
-    for (auto& e : p->deal_cache)
-        if (e.first == S_pad[0]) return e.second;
+    if (total == 1)
+        for (auto& e : p->deal_cache)
+            if (e.first == S_pad[0]) return e.second;
+    const RangePlan own = pass_ranges(plans, n, S_pad);
+    out.sp = own.sp;
+    if (total > 1) {
+        for (int m = 0; m < n; ++m) out.sp[m] = std::max(own.sp[m], least.sp[m]);
+        return out;
+    }
     const int sms = p->num_sms;
     // balanced deal: every CTA gets U/G units; an item then spans at most
     // (tiles - 1) w G / U + 2 CTAs, which must fit the partial slots, and a
@@ -1499,7 +1503,8 @@ int tc_launch(TcPlan* const* plans, int n, TcRun* runs, cudaStream_t st, std::st
     TcRun* srun[kMaxTcModes];
     int64_t S[kMaxTcModes];
     for (int m = 0; m < n; ++m) S[m] = runs[m].S_pad;
-    const RangePlan all = plans[0]->split > 0 ? RangePlan{} : pass_ranges(plans, n, S);
+    RangePlan all;                     // (a lone single-block mode has its deal at hand)
+    if (plans[0]->split == 0 && (n > 1 || plans[0]->nblk > 1)) all = pass_ranges(plans, n, S);
     const bool wide0 = plans[0]->nblk > 1;
     for (int pass = 0; pass < 2; ++pass) {
         int ns = 0;
