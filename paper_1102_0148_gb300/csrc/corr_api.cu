@@ -1188,16 +1188,20 @@ int corr_set_corrections(corr_t h, const float* gains, const float* delays) {
     // two-plane pre-scales and to upload from: one wait for both inputs, none
     // for the uploads.  The inputs may be made by work queued on the handle's
     // stream, where the copies go, or on the legacy default stream, which they
-    // follow.  (Pageable memory is read at once.)
+    // follow.  (Pageable memory is read at once, unless the stream is that one:
+    // then the copies need no look at the pointers.)
     CUDA_TRY(h, cudaEventSynchronize(h->corr_pin_free));   // the previous call's uploads
     float* gh = h->corr_pin;
     float* th = gh + 2 * (size_t)h->N;
-    const bool gp = gains && is_pageable(gains), tp = delays && is_pageable(delays);
+    const bool legacy = !h->stream || h->stream == cudaStreamLegacy;
+    const bool gp = gains && !legacy && is_pageable(gains), tp = delays && !legacy && is_pageable(delays);
     if (gp) memcpy(gh, gains, (size_t)h->N * sizeof(float2));
     if (tp) memcpy(th, delays, (size_t)h->N * sizeof(float));
     if ((gains && !gp) || (delays && !tp)) {
-        CUDA_TRY(h, cudaEventRecord(h->corr_pin_free, cudaStreamLegacy));
-        CUDA_TRY(h, cudaStreamWaitEvent(h->stream, h->corr_pin_free, 0));
+        if (!legacy) {
+            CUDA_TRY(h, cudaEventRecord(h->corr_pin_free, cudaStreamLegacy));
+            CUDA_TRY(h, cudaStreamWaitEvent(h->stream, h->corr_pin_free, 0));
+        }
         if (gains && !gp)
             CUDA_TRY(h, cudaMemcpyAsync(gh, gains, (size_t)h->N * sizeof(float2), cudaMemcpyDefault, h->stream));
         if (delays && !tp)
