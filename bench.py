@@ -61,7 +61,7 @@ NCU_TRAFFIC = {
 # (sm__pipe_tensor_cycles_active.avg.pct_of_peak_sustained_elapsed, summary
 # under profiles/).  Remove an entry when its kernel changes.
 NCU_XENGINE_TENSOR_PCT = {
-    "fp32": 36.38,   # profiles/xengine_tc_n44_k512_onepass_fp32.txt
+    "fp32": 37.02,   # profiles/xengine_tc_n44_k512_onepass_fp32.txt
 }
 
 WORKLOAD = ("N=44 antennas, K=512-point real FFT -> 256 channels, 990 outputs/channel, "
@@ -698,7 +698,7 @@ def measure_precision_form(corr, torch, np, steps=3):
 def measure_batch_form(corr, torch, np, steps=5):
     """Modes (44, 512), (22, 2048), (11, 4096) and the (256, 1024) scale-up,
     2^22 samples per antenna each, in one graph-captured step whose X-engine
-    work is one persistent launch; tiles from a short autotuner sweep.  Error
+    work is two persistent launches; tiles from a short autotuner sweep.  Error
     against the FP64 oracle on a 2^16-sample prefix of every mode."""
     import oracle
     from paper_1102_0148_gb300 import synth, tune

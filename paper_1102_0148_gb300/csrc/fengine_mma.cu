@@ -55,8 +55,9 @@
 //   K = 256,  N = 64,  16384 frames: FP32 mode 4152 -> 230 us, FP16 4099 -> 179
 //             (before: the general radix-2 kernel, one frame at a time);
 //   K = 512,  N = 44,  16384 frames: FP16 337 -> 263 us (unfolded 284), FP8
-//             344 -> 274 (295); FP32 mode 346 against 369 here: the FP32
-//             kernel stays there;
+//             344 -> 274 (295; 294 for the first pass of an integration, whose
+//             first 3072 frames take the FP32 FFT); FP32 mode 346 against 369
+//             here: the FP32 kernel stays there;
 //   K = 1024, N = 256, 4096 frames: FP16 1236 -> 960 us (1130), FP8 977 (1062);
 //             FP32 mode 1374 against 1449 here, the FP32 kernel stays;
 //   K = 2048, N = 64,  4096 frames: FP16 1001 -> 695 us (728), FP8 700 (757),

@@ -391,8 +391,8 @@ __device__ __noinline__ void pair_drain(const PairEnd& e, int rank, int stages, 
 // MMAs are fed (~64 bytes per clock: alone, a CTA's 128 x 256 tile reads 12
 // KB per step and ran at 60% of the tensor rate with its loads taken away),
 // and loads 8 tiles per channel and k-tile at N = 256, not 12.  A pass of
-// 4096 spectra at N = 256, K = 1024: FP32 mode 2033 -> 1393 us, FP16 831 ->
-// 530, FP8 371 -> 275 (with the scales and the issue loop below).
+// 4096 spectra at N = 256, K = 1024: FP32 mode 2033 -> 1402 us, FP16 831 ->
+// 527, FP8 371 -> 264 (with the scales and the issue loop below).
 // Rank 0 issues the MMAs.  Each CTA loads its own tiles, and both CTAs' copies
 // complete on rank 0's full barriers (the loads' .cta_group::2 form), whose
 // phases take the two producers' announcements and all the bytes: rank 0 waits,
